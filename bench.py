@@ -54,7 +54,8 @@ NCU_TRAFFIC = {
 # which layout (kernels, shared device code, launch set-up, tables): a change to any of them
 # voids the stored traffic.
 MEASURED_SOURCES = ("api.cu", "kernels.h", "precompute.cu", "sllbm_internal.cuh", "step_gather.cu",
-                    "step_mapped.cu", "step_uniform.cu", "tma.cuh")
+                    "step_fixup.cu", "step_mapped.cu", "step_uniform.cu", "step_uniform.cuh", "step_uniform_bf16.cu",
+                    "tma.cuh")
 
 
 def _kernel_digest():

@@ -18,9 +18,8 @@ using namespace sllbm;
 enum StepKernel { kKernelUniform = 0, kKernelGather = 1, kKernelPlainF64 = 2, kKernelMapped = 3, kKernelQ9 = 4 };
 constexpr int kXferChunks = 5;   // host transfers move the state in this many plane groups
 // sllbm_step calls of at least kGraphMinSteps steps replay a graph on grids whose state buffer is at
-// most kGraphMaxStateBytes: L2-resident steps are bound by launch overhead.  (On large grids the
-// direct launches are as fast, or faster where the fix-up gather overlaps the fused kernel on
-// its side stream: 0.908 against 0.958 ms a step on the 3073^2 Riemann grid.)
+// most kGraphMaxStateBytes: L2-resident steps are bound by launch overhead.  (On larger grids the
+// direct launches are as fast.)
 constexpr int kGraphMinSteps = 4;
 constexpr size_t kGraphMaxStateBytes = size_t(64) << 20;
 
@@ -39,8 +38,6 @@ struct sllbm_ctx {
   ptrdiff_t ps = 0;
   void* dense = nullptr;                 // dense staging state for host transfers (on demand)
   cudaStream_t xfer = nullptr;           // copy stream of the host transfers (on demand)
-  cudaStream_t side = nullptr;           // fix-up launches beside the fused kernel (on demand)
-  cudaEvent_t side_ev[2] = {};
   cudaGraphExec_t step_graph = nullptr;  // two steps (state 0 -> 1 -> 0), captured on demand
   bool graph_off = false;                // the stream cannot be captured: steps launch directly
   cudaEvent_t xev[kXferChunks + 1] = {};
@@ -63,7 +60,10 @@ struct sllbm_ctx {
   int offx_lo = 0, offx_hi = 0, offy_lo = 0, offy_hi = 0;
   UniformTables ut{};
   unsigned char *std_x = nullptr, *std_y = nullptr;
-  int* fix_list = nullptr;       // vertices the fused kernels leave to the gather kernel
+  float4* etail[2] = {nullptr, nullptr};         // per-vertex stencils of the x and y axis (edge tiles)
+  unsigned char* ebef[2] = {nullptr, nullptr};
+  int2* edge_tiles = nullptr;
+  int* fix_list = nullptr;       // vertices the fused kernels leave to the fix-up (uniform) or gather (mapped) kernel
   long long n_fix = 0;
   // mapped-grid tiles
   MappedTables mt{};
@@ -210,6 +210,8 @@ static void gauss_legendre01(int n, double* x, double* w) {
   }
 }
 
+static size_t dense_bytes(const sllbm_ctx* c) { return (size_t)c->npop * c->nq * c->nv * c->elem; }
+
 static StepArgs step_args(sllbm_ctx* c, const void* src, void* dst) {
   StepArgs a{};
   a.src = src;
@@ -274,8 +276,20 @@ static GeomArgs geom_args(sllbm_ctx* c) {
 // taken from a cell in the middle of each axis; a vertex "follows the pattern" when its offset
 // and weights match those of its local node for all five components.  The fused kernel writes
 // only vertices that follow the pattern on both axes; the others go to the gather kernel.
+// Every vertex's own stencil is kept too, as the fused kernel's edge tiles read it: tail sums of the
+// weights and whether it is the cell before the vertex's own (whole: all stencils are one of the
+// two).
+struct AxisPattern {
+  std::vector<unsigned char> follows;   // [n]
+  std::vector<float4> tail;             // [5][n]: W_1..W_P, W_alpha = sum_{beta >= alpha} w_beta
+  std::vector<unsigned char> before;    // [5][n]
+  bool whole = true;
+  int lo = 0, hi = 0;                   // the run of vertices around the middle that follow the pattern
+};
+
 static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const int* off_dev, const double* w_dev,
-                                 bool is_y, std::vector<unsigned char>& stdv, bool* ok) {
+                                 bool is_y, AxisPattern& pat, bool* ok) {
+  std::vector<unsigned char>& stdv = pat.follows;
   const int n = ax.nv, P = c->P;
   std::vector<int> off((size_t)kQ1 * n);
   std::vector<double> w((size_t)kQ1 * n * (P + 1));
@@ -311,6 +325,24 @@ static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const int* off_d
       if (!same) stdv[j] = 0;
     }
   }
+  pat.tail.resize((size_t)kQ1 * n);
+  pat.before.resize((size_t)kQ1 * n);
+  for (int comp = 0; comp < kQ1; ++comp)
+    for (int j = 0; j < n; ++j) {
+      const size_t e = (size_t)comp * n + j;
+      float tail[4] = {0.f, 0.f, 0.f, 0.f};
+      double acc = 0.0;
+      for (int al = P; al >= 1; --al) {
+        acc += w[e * (P + 1) + al];
+        tail[al - 1] = (float)acc;
+      }
+      pat.tail[e] = make_float4(tail[0], tail[1], tail[2], tail[3]);
+      pat.before[e] = j % P == 0 && off[e] == -P;
+      if (!pat.before[e] && off[e] != -(j % P)) pat.whole = false;
+    }
+  pat.lo = pat.hi = jref0;
+  while (pat.lo > 0 && stdv[pat.lo - 1]) --pat.lo;
+  while (pat.hi < n && stdv[pat.hi]) ++pat.hi;
   return SLLBM_OK;
 }
 
@@ -318,12 +350,13 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c) {
   c->ut.valid = false;
   // Any vertex count: the tensor copies start on 16-byte boundaries of the padded rows whatever nx
   // is, and the ghost cells carry the periodic seam.  (Periodic axes of nx % 4 != 0 took the gather
-  // kernel before: 1.13 ms a step on 1023 x 1023 vertices of order 3, 0.107 ms here.)
+  // kernel before: 1.13 ms a step on 1023 x 1023 vertices of order 3, 0.106 ms here.)
   if (c->xs != 2) return SLLBM_OK;
-  std::vector<unsigned char> sx, sy;
+  AxisPattern px, py;
+  const std::vector<unsigned char>&sx = px.follows, &sy = py.follows;
   bool okx = false, oky = false;
-  TRY(axis_pattern(c, c->ax, c->offx, c->wx64, false, sx, &okx));
-  TRY(axis_pattern(c, c->ay, c->offy, c->wy64, true, sy, &oky));
+  TRY(axis_pattern(c, c->ax, c->offx, c->wx64, false, px, &okx));
+  TRY(axis_pattern(c, c->ay, c->offy, c->wy64, true, py, &oky));
   if (!okx || !oky) return SLLBM_OK;
   // The fused kernel takes each stencil as a whole cell, on both axes: start offset -l at local
   // node l, or -P at node 0 (a departure into the cell before).  Anything else goes to the
@@ -340,10 +373,44 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c) {
   }
   CUDA_TRY(c, cudaMemcpy(c->std_x, sx.data(), sx.size(), cudaMemcpyHostToDevice));
   CUDA_TRY(c, cudaMemcpy(c->std_y, sy.data(), sy.size(), cudaMemcpyHostToDevice));
+  // Vertices off the pattern, next to zero-gradient boundaries.  On states beyond the L2 a second
+  // launch of the fused kernel does the tiles that hold them: gathered one by one from HBM, each
+  // of the 25 planes of a boundary column touches pages of its own (3073^2 vertices, p = 3: 0.857 ms
+  // a step so, 0.905 ms with the fix-up kernel).  On states in the L2 the fix-up kernel's single
+  // gather per warp is the shorter one (8193 x 8, p = 2: 17.5 us a step, 18.4 us with edge tiles).
+  const bool uneven = px.lo > 0 || px.hi < c->nx || py.lo > 0 || py.hi < c->ny;
+  c->ut.edge = uneven && px.whole && py.whole && dense_bytes(c) > kGraphMaxStateBytes;
+  if (c->ut.edge) {
+    if (!c->etail[0]) {
+      TRY(dalloc(c, &c->etail[0], px.tail.size()));
+      TRY(dalloc(c, &c->etail[1], py.tail.size()));
+      TRY(dalloc(c, &c->ebef[0], px.before.size()));
+      TRY(dalloc(c, &c->ebef[1], py.before.size()));
+    }
+    for (int k = 0; k < 2; ++k) {
+      const AxisPattern& pat = k ? py : px;
+      CUDA_TRY(c, cudaMemcpy(c->etail[k], pat.tail.data(), pat.tail.size() * sizeof(float4), cudaMemcpyHostToDevice));
+      CUDA_TRY(c, cudaMemcpy(c->ebef[k], pat.before.data(), pat.before.size(), cudaMemcpyHostToDevice));
+    }
+    c->ut.tail_x = c->etail[0];
+    c->ut.tail_y = c->etail[1];
+    c->ut.bef_x = c->ebef[0];
+    c->ut.bef_y = c->ebef[1];
+    c->ut.px0 = px.lo;
+    c->ut.px1 = px.hi;
+    c->ut.py0 = py.lo;
+    c->ut.py1 = py.hi;
+    std::vector<int2> tiles;
+    uniform_edge_tiles(c->P, c->nx, c->ny, c->ut, tiles);
+    if (!c->edge_tiles) TRY(dalloc(c, &c->edge_tiles, tiles.size()));
+    CUDA_TRY(c, cudaMemcpy(c->edge_tiles, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    c->ut.edge_tiles = c->edge_tiles;
+  }
   std::vector<int> fix;
-  for (int iy = 0; iy < c->ny; ++iy)
-    for (int ix = 0; ix < c->nx; ++ix)
-      if (!sx[ix] || !sy[iy]) fix.push_back(iy * c->nx + ix);
+  if (uneven && !c->ut.edge)
+    for (int iy = 0; iy < c->ny; ++iy)
+      for (int ix = 0; ix < c->nx; ++ix)
+        if (!sx[ix] || !sy[iy]) fix.push_back(iy * c->nx + ix);
   c->n_fix = (long long)fix.size();
   if (!fix.empty()) {
     TRY(dalloc(c, &c->fix_list, fix.size()));
@@ -354,6 +421,7 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c) {
   c->ut.gx = c->gx;
   c->ut.gy = c->gy;
   c->ut.rows_alloc = c->rows_alloc;
+  c->ut.fixup = c->n_fix > 0;
   c->ut.valid = true;
   return SLLBM_OK;
 }
@@ -522,8 +590,6 @@ static cudaError_t convert_pairs(sllbm_ctx* c, const void* src, void* dst, bool 
                              c->plane_stride, c->stream);
 }
 
-static size_t dense_bytes(const sllbm_ctx* c) { return (size_t)c->npop * c->nq * c->nv * c->elem; }
-
 // Dense [npop][nq][ny][nx] state (host or device) <-> the internal layout.  Host transfers go in
 // kXferChunks groups of planes on a copy stream, each group's conversion on the compute stream
 // overlapping the next group's copy.  With (f, g) pairs a group is a range of velocity planes
@@ -627,12 +693,6 @@ sllbm_status sllbm_destroy(sllbm_ctx* c) {
   if (c->step_graph) {
     cudaStreamSynchronize(c->stream);
     cudaGraphExecDestroy(c->step_graph);
-  }
-  if (c->side) {
-    cudaStreamSynchronize(c->side);
-    cudaStreamDestroy(c->side);
-    for (int k = 0; k < 2; ++k)
-      if (c->side_ev[k]) cudaEventDestroy(c->side_ev[k]);
   }
   if (c->xfer) {
     cudaStreamSynchronize(c->xfer);
@@ -886,38 +946,18 @@ sllbm_status sllbm_init_equilibrium(sllbm_ctx* c, const double* rho, const doubl
   return SLLBM_OK;
 }
 
-// The side stream and its two events of the fix-up gather (created on first use).
-static cudaError_t ensure_side(sllbm_ctx* c) {
-  if (c->side) return cudaSuccess;
-  cudaError_t e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-  for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaEventCreateWithFlags(&c->side_ev[k], cudaEventDisableTiming);
-  return e;
-}
-
 static cudaError_t enqueue_step(sllbm_ctx* c, float* mom = nullptr) {
   StepArgs a = step_args(c, c->state[c->cur], c->state[c->cur ^ 1]);
   a.mom = mom;
   cudaError_t e;
   switch (c->kernel) {
     case kKernelUniform:
-      if (c->n_fix > 0) {
-        // vertices off the cell-periodic pattern: the gather kernel reads the same source and
-        // writes other vertices than the fused kernel, so it runs on a side stream beside it
-        // (filling the SMs the persistent kernel's tail leaves idle); the step ends when both do
-        if ((e = ensure_side(c)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(c->side_ev[0], c->stream)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(c->side, c->side_ev[0], 0)) != cudaSuccess) return e;
-        e = launch_step_uniform(a, c->ut, c->store, c->stream);
-        if (e != cudaSuccess) return e;
-        StepArgs f = a;
-        f.vlist = c->fix_list;
-        f.nlist = c->n_fix;
-        f.mapped = 0;
-        if ((e = launch_step_gather(f, c->store, c->side)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(c->side_ev[1], c->side)) != cudaSuccess) return e;
-        e = cudaStreamWaitEvent(c->stream, c->side_ev[1], 0);
-      } else {
-        e = launch_step_uniform(a, c->ut, c->store, c->stream);
+      e = launch_step_uniform(a, c->ut, c->store, c->stream);
+      if (e == cudaSuccess && c->n_fix > 0) {   // vertices off the cell-periodic pattern
+        a.vlist = c->fix_list;
+        a.nlist = c->n_fix;
+        a.mapped = 0;
+        e = launch_step_fixup(a, c->store, c->stream);
       }
       break;
     case kKernelMapped:
@@ -938,12 +978,9 @@ static cudaError_t enqueue_step(sllbm_ctx* c, float* mom = nullptr) {
 }
 
 // A CUDA graph of two steps, from state buffer 0 through 1 back to 0: every launch of the steps
-// (the fused kernel, the fix-up gather on its side stream and the events between them) with its
-// parameters as the step's host set-up computed them.  The buffers and tables it refers to live
-// as long as the context, so the graph stays valid.
+// (the fused kernel, the fix-up beside it) with its parameters as the step's host set-up computed
+// them.  The buffers and tables it refers to live as long as the context, so the graph stays valid.
 static cudaError_t build_step_graph(sllbm_ctx* c) {
-  cudaError_t e = ensure_side(c);   // nothing is created while capturing
-  if (e != cudaSuccess) return e;
   if (c->stream == nullptr || c->stream == cudaStreamLegacy ||
       cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
     cudaGetLastError();   // the legacy default stream (or another one capture refuses): no graph
@@ -954,7 +991,7 @@ static cudaError_t build_step_graph(sllbm_ctx* c) {
   cudaError_t e1 = enqueue_step(c);
   if (e1 == cudaSuccess) e1 = enqueue_step(c);
   cudaGraph_t g = nullptr;
-  e = cudaStreamEndCapture(c->stream, &g);
+  cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   c->cur = cur0;   // the captured steps did not run
   if (e1 != cudaSuccess || e != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
@@ -1006,7 +1043,9 @@ const char* sllbm_step_kernel_name(const sllbm_ctx* c) {
 
 int sllbm_launches_per_step(const sllbm_ctx* c) {
   if (!c) return 0;
-  return ((c->kernel == kKernelUniform || c->kernel == kKernelMapped) && c->n_fix > 0) ? 2 : 1;
+  return ((c->kernel == kKernelUniform || c->kernel == kKernelMapped) && c->n_fix > 0) ||
+                 (c->kernel == kKernelUniform && c->ut.edge && c->ut.in_x1 > c->ut.in_x0)
+             ? 2 : 1;
 }
 
 

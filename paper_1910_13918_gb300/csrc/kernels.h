@@ -3,6 +3,8 @@
 
 #include <stddef.h>
 
+#include <vector>
+
 #include "sllbm_internal.cuh"
 
 namespace sllbm {
@@ -66,6 +68,17 @@ struct UniformTables {
   const unsigned char* std_x; // [nx]: column follows the pattern
   const unsigned char* std_y; // [ny]
   int gx, gy, rows_alloc;     // ghost columns/rows before the interior origin; rows per plane
+  bool fixup;                 // launch_step_fixup follows on the same stream
+  // edge: a second launch of the fused kernel takes the tiles with vertices off the pattern
+  // (edge_tiles), from the per-vertex stencils of both axes ([5][n]: tail sums W_1..W_P; 1 if the
+  // stencil is the cell before); columns [px0, px1) and rows [py0, py1) follow the pattern, and the
+  // tiles [in_x0, in_x1) x [in_y0, in_y1) lie within
+  bool edge;
+  const int2* edge_tiles;
+  int n_edge, in_x0, in_x1, in_y0, in_y1;
+  const float4 *tail_x, *tail_y;
+  const unsigned char *bef_x, *bef_y;
+  int px0, px1, py0, py1;
 };
 
 // Fused shared-memory step for mapped grids: per (tile of kMappedTileX x kMappedTileY vertices,
@@ -90,8 +103,14 @@ size_t mapped_smem_bytes(int bw, int bh, int store);
 // Generic FP32 gather step (one thread per vertex, (p+1)^2 gathers per plane from L1/L2).
 cudaError_t launch_step_gather(const StepArgs& a, int store, cudaStream_t s);
 // Fused shared-memory step for uniform grids (pattern band interpolation); writes only the
-// vertices marked in std_x/std_y.  cudaErrorNotSupported if the tables are not valid.
+// vertices marked in std_x/std_y, or with t.edge every vertex in two launches.  cudaErrorNotSupported if the tables are not valid.
 cudaError_t launch_step_uniform(const StepArgs& a, const UniformTables& t, int store, cudaStream_t s);
+// The listed vertices (vlist, nlist) of a uniform grid, one warp per vertex: those the fused uniform
+// kernel leaves out.  Launched on the same stream right after that kernel, it runs beside its end.
+cudaError_t launch_step_fixup(const StepArgs& a, int store, cudaStream_t s);
+// The tiles of the fused kernel that hold vertices off the pattern, from t.px0 .. t.py1; sets
+// t.n_edge and the rectangle in between.
+void uniform_edge_tiles(int P, int nx, int ny, UniformTables& t, std::vector<int2>& tiles);
 // Plain FP64 step on full populations.
 cudaError_t launch_step_plain_f64(const StepArgs& a, cudaStream_t s);
 // D2Q9 step (isothermal, one population, planar storage): FP32 arithmetic on FP32/BF16

@@ -1,8 +1,10 @@
 """Uniform grids at the edges of the fused kernel's range: periodic axes whose vertex counts are no
-multiple of 4 (down to three cells), and the fix-up of the vertices next to
+multiple of 4 (down to three cells), and the warp-per-vertex fix-up of the vertices next to
 zero-gradient boundaries with every option it carries (storage, Prandtl number, one population,
 the isothermal equilibrium, the moments epilogue).  FP32 against the oracle at the tolerances of
-the other parity tests: 1e-5 after one step, 1e-4 after 30."""
+the other parity tests: 1e-5 after one step, 1e-4 after 30.  On states larger than the L2 (over
+64 MB) the edge-tile launch takes those vertices: one step against the plain FP64 step from the
+same state, every value within 2e-6 (about 30 FP32 roundings of values below 1)."""
 import dataclasses
 
 import numpy as np
@@ -65,3 +67,34 @@ def test_edges_moments_epilogue(gpu_lib, name):
     for k, key in enumerate(("rho", "u", "v", "T")):
         a, b = mom[k].cpu().numpy().astype(np.float64), m[key].cpu().numpy().astype(np.float64)
         assert np.max(np.abs(a - b)) <= 3e-6 * max(1.0, np.max(np.abs(b))), (name, key)
+
+
+LARGE = {   # over 335,544 vertices: 50 FP32 values a vertex are more than 64 MB
+    "p1_clamped": _tgv(1, 600, 577, bc=(ZG, ZG)), "p2_clamped_y": _tgv(2, 301, 300, bc=(PER, ZG)),
+    "p3_clamped_x": _tgv(3, 197, 200, bc=(ZG, PER)), "p3_clamped_pr": _tgv(3, 200, 191, bc=(ZG, ZG), pr=0.75),
+    "p4_clamped": _tgv(4, 151, 147, bc=(ZG, ZG)), "p4_strip": _tgv(4, 20000, 4, bc=(ZG, ZG)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(LARGE))
+def test_edge_tiles_against_the_plain_step(gpu_lib, name):
+    from paper_1910_13918_gb300.sllbm import SLLBM
+    w = LARGE[name]
+    a, b = SLLBM.from_workload(w, prec="f32"), SLLBM.from_workload(w, prec="f64")
+    for s in (a, b):
+        s.precompute()
+    x, y = (t.cpu().numpy() for t in a.coords())
+    a.init(*w.fields(x, y, perturb=True))
+    lat = np.outer(*[np.array(H.o.d1q5()[1])] * 2).reshape(-1)
+    full = a.get_state().double()
+    for k, c in enumerate((1.0, 2 * w.cv - 2)):
+        full[k] += c * full.new_tensor(lat)[:, None, None]
+    b.set_state(full)
+    a.step(1)
+    b.step(1)
+    got, ref = a.get_state().double(), b.get_state()
+    for k, c in enumerate((1.0, 2 * w.cv - 2)):
+        ref[k] -= c * ref.new_tensor(lat)[:, None, None]
+    err = float((got - ref).abs().max())
+    assert (a.kernel_name, a.launches_per_step) == ("uniform_fused", 2)
+    assert err <= 2e-6, (name, err)
