@@ -258,8 +258,10 @@ __global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__
   // theta - 1 = (A2 + G - rho |u|^2 - 2 C_v drho) / (2 C_v rho)   (sum w |xi|^2 + K = 2 C_v)
   const float qk = (a2 + G - rho * (ux * ux + uy * uy + uz * uz) - 2.f * a.cv * drho) * inv_rho * a.inv2cv;
   const float q = a.iso ? 0.f : qk;
-  // per-axis factors X_k(a) = A_k(u_x) he_k(a), Y_l(b) likewise, Zc_n(c) = sum_{m <= n} A_m(u_z)
-  // he_m(c): 1 + S_abc = sum_{k + l + m <= 4} X_k(a) Y_l(b) Z_m(c), and f^eq - w = w (drho + rho S)
+  // per-axis factors X_k(a) = A_k(u_x) he_k(a), Y_l(b) likewise, and Zc_n(c) = sum_{1 <= m <= n}
+  // A_m(u_z) he_m(c): S_abc = sum_{k + l + m <= 4} X_k(a) Y_l(b) Z_m(c) - 1 = sum_n C_n (1 + Zc_n(c)) - 1
+  // with C_n = sum_{k + l = 4 - n} X_k(a) Y_l(b), C_4 = 1, without forming the leading 1; and
+  // f^eq - w = w (drho + rho S)
   float Ax[5], Ay[5], Az[5];
   {
     const float u3[3] = {ux, uy, uz};
@@ -278,8 +280,9 @@ __global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     float acc = 0.f;
+    Zc[0][c] = 0.f;
 #pragma unroll
-    for (int m = 0; m < 5; ++m) {
+    for (int m = 1; m < 5; ++m) {
       acc += Az[m] * a.cs.hef[m][c];
       Zc[m][c] = acc;
     }
@@ -299,19 +302,16 @@ __global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__
 #pragma unroll
       for (int l = 0; l < 5; ++l) Yb[l] = Ay[l] * a.cs.hef[l][ib];
       const float ey = a.cs.xif[ib], wab = wa * a.cs.wf[ib];
+      const float C3 = Xa[1] + Yb[1], C2 = Xa[2] + Yb[2] + Xa[1] * Yb[1],
+                  C1 = Xa[3] + Yb[3] + Xa[2] * Yb[1] + Xa[1] * Yb[2],
+                  C0 = Xa[4] + Yb[4] + Xa[3] * Yb[1] + Xa[1] * Yb[3] + Xa[2] * Yb[2];
+      const float Cs = C0 + C1 + C2 + C3;
 #pragma unroll
       for (int ic = 0; ic < kQ1; ++ic) {
         const int i = 25 * ia + 5 * ib + ic;
-        float s1 = 0.f;
-#pragma unroll
-        for (int k = 0; k <= 4; ++k) {
-          float sl = 0.f;
-#pragma unroll
-          for (int l = 0; l <= 4 - k; ++l) sl += Yb[l] * Zc[4 - k - l][ic];
-          s1 += Xa[k] * sl;
-        }
+        const float em1 = fmaf(C1, Zc[1][ic], fmaf(C2, Zc[2][ic], fmaf(C3, Zc[3][ic], Cs + Zc[4][ic])));
         const float w = wab * a.cs.wf[ic];
-        const float ef = w * (drho + rho * (s1 - 1.f));
+        const float ef = w * fmaf(rho, em1, drho);
         const float eg = Kq1 * ef + Kq * w;   // g^eq - K w = K ((1 + q)(f^eq - w) + q w)
         float2* o = a.dst + (size_t)i * plane + v;
         const float2 fg = *o;
@@ -348,14 +348,12 @@ __global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__
   if (!((rho > 0.f) && (qk > -1.f) && isfinite(rho) && isfinite(qk))) atomicOr(a.flag, 1);
 }
 
-// ---- sum-factorised FP32 step (orders 1 and 2; an even number of x vertices, so that the
-// pair rows are whole 16-byte units for the tensor copies) ----
+// ---- sum-factorised FP32 step ----
 //
-// Three launches a step.  stream3d_kernel: a CTA takes a tile of 32 x 8 x 4 vertices (two CTAs
-// an SM) and walks the
+// Two launches a step.  stream3d_kernel: a CTA takes a tile of 32 x 8 x TZ vertices and walks the
 // 125 velocity planes; per plane one TMA tensor copy brings the source region (the tile and the
-// stencil halo: x0 - 2 .. x0 + 33, and p on both sides in y and z), one plane ahead in two
-// stages.  The state keeps 2 ghost cells on every axis, holding the periodic images on periodic
+// stencil halo: XO = p rounded up to even columns on both sides in x, p in y and z) into a ring of
+// NS stages.  The state keeps ghost cells on every axis, holding the periodic images on periodic
 // axes (zero, and never read by an interior vertex, on zero-gradient ones), so a region never
 // wraps.  The interpolation is sum-factorised: z pass over the region's (y, x) columns, y pass
 // over the tile's z and the region's x, x pass into the destination, each in a centred tail-sum
@@ -363,29 +361,50 @@ __global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__
 //   sum_d W_d v_{c+d} = v_c + sum_{j=1..p} T+_j (v_{c+j} - v_{c+j-1}) - sum_{j=1..p} T-_j (v_{c-j+1} - v_{c-j}),
 //   T+_j = sum_{d >= j} W_d, T-_j = sum_{d <= -j} W_d  (d the offset from the vertex, W_d its weight),
 // equal to the Lagrange sum because the weights sum to one and exact for constant fields in FP32.
-// The tile's tail sums of all five components are loaded once.  The thread of a vertex in the x
-// pass sums its moments over the 125 planes.  collide3d_kernel then relaxes every vertex's 125
-// pairs in place and writes the periodic images of the vertices next to periodic faces.
-constexpr int kT3X = 32, kT3Y = 8, kT3Z = 4, kT3NT = 256;
-constexpr int kT3XO = 2;   // the region starts at x0 - 2: 16-byte aligned for both orders
-constexpr int kT3G = 2;    // ghost cells of the state on every axis (>= the halo of p <= 2)
+// The passes are pipelined over the planes: phase i runs the z pass of plane i, the y pass of plane
+// i - 1 and the x pass of plane i - 2, on double-buffered results, so a phase has one barrier and
+// three independent pieces of work in place of three dependent ones with a barrier each.  In the x
+// pass a thread takes two neighbouring vertices: their common window comes in 16-byte loads, and
+// the two results leave in one 16-byte store.  The thread sums its vertices' moments over the 125
+// planes.  collide3d_kernel then relaxes every vertex's 125 pairs in place and writes the periodic
+// images of the vertices next to periodic faces.
+//
+// What bounds it: the latency of the phases and shared memory together (64^3: the LSU pipe at 65 %,
+// issue at 39 %; 128^3: 1.205 ms, 1.38 ms with three barriers a plane and one vertex a task).  Deeper
+// tiles (32 x 8 x 8, three stages, one CTA of 512 threads) take the same time; 24 warps an SM on
+// tiles of 3 or 2 slices take 1.50 and 1.44 ms, as their regions grow.  250 values a vertex rule out a
+// collision in registers, so the two kernels move 16 bytes an update.
+constexpr int kT3X = 32, kT3Y = 8;
+
+// Tile depth, threads and stages by order.
+template <int P>
+struct T3Config {
+  static constexpr int TZ = 4, NT = P <= 2 ? 256 : 512, NS = 2, MINB = P <= 2 ? 2 : 1;
+};
 
 template <int P>
 struct T3Shape {
-  static constexpr int RX = kT3X + 2 * kT3XO, RY = kT3Y + 2 * P, RZ = kT3Z + 2 * P;
+  using C = T3Config<P>;
+  static constexpr int TZ = C::TZ, NT = C::NT, NS = C::NS;
+  static constexpr int XO = (P + 1) / 2 * 2;   // the region starts at x0 - XO: 16-byte aligned
+  static constexpr int RX = kT3X + 2 * XO, RY = kT3Y + 2 * P, RZ = TZ + 2 * P;
   static constexpr int RE = RX * RY * RZ;   // region pairs
   static constexpr int NW = 2 * P;          // tail sums per (component, node): T+_1..p, -T-_1..p
   static constexpr int ZT = RY * RX;        // z-pass columns
-  static constexpr int YT = kT3Z * RX;      // y-pass columns
-  static constexpr int NWT = kQ1 * (kT3Z + kT3Y + kT3X) * NW;   // the tile's tail sums
+  static constexpr int YT = TZ * RX;        // y-pass columns
+  // slices of the z and y results, padded so that the columns of a warp that crosses from one slice
+  // to the next go on over the shared-memory banks as in one row (16 pairs)
+  static constexpr int ZS = RY * RX + ((RX - RY * RX) % 16 + 16) % 16, YS = kT3Y * RX + ((RX - kT3Y * RX) % 16 + 16) % 16;
+  static constexpr int ZB = TZ * ZS, YB = TZ * YS;   // pairs of one z / y result
+  static constexpr int NWT = kQ1 * (TZ + kT3Y + kT3X) * NW;   // the tile's tail sums
   static constexpr size_t kStage = sizeof(float2) * RE;
-  static constexpr size_t kBytes = 128 + 2 * kStage +
-                                   sizeof(float2) * (size_t)(kT3Z * RY * RX + kT3Z * kT3Y * RX) +
-                                   sizeof(float) * NWT + sizeof(uint64_t) * 2;
-  static_assert(kStage % 128 == 0, "stages stay 128-byte aligned");
-  static constexpr int XR = kT3Y * kT3Z / (kT3NT / 32);   // x-pass rows per warp
-  static_assert(YT <= kT3NT && XR * (kT3NT / 32) == kT3Y * kT3Z, "one y column a thread, whole x rows a warp");
-  static_assert(P <= kT3G && kT3XO <= kT3G, "the halo stays within the ghost cells");
+  static constexpr size_t kStride = (kStage + 127) / 128 * 128;
+  static constexpr size_t kBytes = 128 + NS * kStride + sizeof(float2) * 2 * (size_t)(ZB + YB) +
+                                   sizeof(float) * NWT + sizeof(uint64_t) * NS;
+  static constexpr int XT = kT3X / 2 * kT3Y * TZ / NT;   // x-pass tasks (two vertices each) per thread
+  static_assert(YT <= NT && XT * NT == kT3X / 2 * kT3Y * TZ, "one y column a thread at most, x tasks split evenly");
+  static_assert((sizeof(float2) * (ZB + YB)) % 16 == 0 && NWT % 2 == 0, "16-byte rows, 8-byte barriers");
+  static constexpr int G = XO;   // ghost cells of the state on every axis
 };
 
 struct Stream3Args {
@@ -415,163 +434,231 @@ __device__ __forceinline__ float2 tail_interp(const float2 (&v)[N], const float2
 }
 
 template <int P>
-__global__ void __launch_bounds__(kT3NT, 2) stream3d_kernel(const __grid_constant__ Stream3Args a,
-                                                            const __grid_constant__ CUtensorMap smap) {
+__global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
+    stream3d_kernel(const __grid_constant__ Stream3Args a, const __grid_constant__ CUtensorMap smap) {
   using SH = T3Shape<P>;
-  constexpr int RX = SH::RX, RY = SH::RY, RZ = SH::RZ, RE = SH::RE, NW = SH::NW;
+  constexpr int TZ = SH::TZ, NT = SH::NT, NS = SH::NS, XO = SH::XO;
+  constexpr int RX = SH::RX, RY = SH::RY, RZ = SH::RZ, NW = SH::NW, XT = SH::XT;
   extern __shared__ unsigned char s3_smem[];
   unsigned char* base = s3_smem + ((128 - (smem_u32(s3_smem) & 127)) & 127);
-  float2* S = reinterpret_cast<float2*>(base);                         // [2][RZ][RY][RX]
-  float2* Zb = S + 2 * RE;                                             // [TZ][RY][RX]
-  float2* Yb = Zb + kT3Z * RY * RX;                                    // [TZ][TY][RX]
-  float* Wz = reinterpret_cast<float*>(Yb + kT3Z * kT3Y * RX);         // [5][TZ][NW]
-  float* Wy = Wz + kQ1 * kT3Z * NW;                                    // [5][TY][NW]
+  float2* Zb = reinterpret_cast<float2*>(base + NS * SH::kStride);      // [2][TZ][RY][RX] (slices ZS apart), after the stages
+  float2* Yb = Zb + 2 * SH::ZB;                                        // [2][TZ][TY][RX] (slices YS apart)
+  float* Wz = reinterpret_cast<float*>(Yb + 2 * SH::YB);               // [5][TZ][NW]
+  float* Wy = Wz + kQ1 * TZ * NW;                                      // [5][TY][NW]
   float* Wx = Wy + kQ1 * kT3Y * NW;                                    // [5][TX][NW]
-  uint64_t* BAR = reinterpret_cast<uint64_t*>(Wx + kQ1 * kT3X * NW);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint64_t* BAR = reinterpret_cast<uint64_t*>(Wx + kQ1 * kT3X * NW);   // [NS]
+  const int tid = threadIdx.x;
   const int tiles_x = (a.nx + kT3X - 1) / kT3X, tiles_y = (a.ny + kT3Y - 1) / kT3Y;
   const int byz = (int)blockIdx.x / tiles_x;
   const int x0 = ((int)blockIdx.x - byz * tiles_x) * kT3X, y0 = (byz % tiles_y) * kT3Y,
-            z0 = (byz / tiles_y) * kT3Z;
+            z0 = (byz / tiles_y) * TZ;
   // the tile's tail sums of all components (nodes past the grid clamped: those outputs are not
   // stored)
-  for (int e = tid; e < SH::NWT; e += kT3NT) {
+  for (int e = tid; e < SH::NWT; e += NT) {
     const int q = e % NW, r = e / NW;
     float t;
-    if (r < kQ1 * kT3Z) {
-      const int c = r / kT3Z, n = min(z0 + r - c * kT3Z, a.nz - 1);
+    if (r < kQ1 * TZ) {
+      const int c = r / TZ, n = min(z0 + r - c * TZ, a.nz - 1);
       t = __ldg(a.tz + ((size_t)c * a.nz + n) * NW + q);
-    } else if (r < kQ1 * (kT3Z + kT3Y)) {
-      const int r2 = r - kQ1 * kT3Z, c = r2 / kT3Y, n = min(y0 + r2 - c * kT3Y, a.ny - 1);
+    } else if (r < kQ1 * (TZ + kT3Y)) {
+      const int r2 = r - kQ1 * TZ, c = r2 / kT3Y, n = min(y0 + r2 - c * kT3Y, a.ny - 1);
       t = __ldg(a.ty + ((size_t)c * a.ny + n) * NW + q);
     } else {
-      const int r2 = r - kQ1 * (kT3Z + kT3Y), c = r2 / kT3X, n = min(x0 + r2 - c * kT3X, a.nx - 1);
+      const int r2 = r - kQ1 * (TZ + kT3Y), c = r2 / kT3X, n = min(x0 + r2 - c * kT3X, a.nx - 1);
       t = __ldg(a.tx + ((size_t)c * a.nx + n) * NW + q);
     }
     Wz[e] = t;   // Wz, Wy and Wx are consecutive
   }
   if (tid == 0) {
-    mbar_init(&BAR[0], 1);
-    mbar_init(&BAR[1], 1);
+    for (int k = 0; k < NS; ++k) mbar_init(&BAR[k], 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   __syncthreads();
-  // region origin in the ghost-padded layout: x0 - 2 + g (x in floats: 2 (x0 - 2 + g), a multiple
-  // of 4, i.e. 16 bytes), y0 - p + g, z0 - p + g
-  const int cx = 2 * (x0 - kT3XO + a.lay.g), cy = y0 - P + a.lay.g, cz = z0 - P + a.lay.g;
+  // region origin in the ghost-padded layout (g = XO): x0 (x in floats: 2 x0, a multiple of 4, i.e.
+  // 16 bytes), y0 - p + g, z0 - p + g
+  const int cx = 2 * (x0 - XO + a.lay.g), cy = y0 - P + a.lay.g, cz = z0 - P + a.lay.g;
   auto issue = [&](int i, int st) {   // thread 0: plane i into stage st
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     mbar_expect_tx(&BAR[st], (unsigned)SH::kStage);
-    tma_load_4d(S + (size_t)st * RE, &smap, cx, cy, cz, i, &BAR[st]);
+    tma_load_4d(base + (size_t)st * SH::kStride, &smap, cx, cy, cz, i, &BAR[st]);
   };
-  if (tid == 0) issue(0, 0);
-  // x pass: warp w takes the tile rows XR w .. XR w + XR - 1 (row r: z = r / TY, y = r % TY),
-  // lane = x
-  constexpr int XR = SH::XR;
-  const int vx = x0 + lane;
-  float m[XR][6];
+  if (tid == 0)
+    for (int k = 0; k < NS - 1; ++k) issue(k, k);
+  // y pass: this thread's column (tz, rx); the last threads of the CTA, as the first ones have the
+  // most z columns
+  const int yt = tid - (NT - SH::YT);
+  const int ytz = yt < 0 ? 0 : yt / RX, ycol = yt < 0 ? 0 : yt - ytz * RX;
+  // x pass: task r = tid + k NT is the vertices x0 + 2 (r % 16) and the next one of tile row
+  // r / 16 (z = row / TY, y = row % TY)
+  const int xp = tid & 15;
+  const int vx = x0 + 2 * xp;
+  float2* out[XT];   // destination of the tasks, advancing plane by plane
+  bool on[XT];
 #pragma unroll
-  for (int j = 0; j < XR; ++j)
+  for (int k = 0; k < XT; ++k) {
+    const int row = (tid + k * NT) >> 4, vy = y0 + row % kT3Y, vz = z0 + row / kT3Y;
+    on[k] = vx < a.nx && vy < a.ny && vz < a.nz;
+    out[k] = a.dst + a.lay.at(0, vx, vy, vz);
+  }
+  const bool both = vx + 1 < a.nx;   // an odd x count ends with half a task
+  // per vertex: (sum f, sum g), sum f xi_y, sum f xi_z, sum f (xi_y^2 + xi_z^2); over the planes of
+  // one x component (f alone), and over all
+  float2 fg[XT][2], part[XT][2];
+  float my[XT][2], mz[XT][2], m2[XT][2], mx[XT][2];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) m[j][q] = 0.f;
-  float wx[NW];
+  for (int k = 0; k < XT; ++k)
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      fg[k][v] = part[k][v] = make_float2(0.f, 0.f);
+      my[k][v] = mz[k][v] = m2[k][v] = mx[k][v] = 0.f;
+    }
+  float wx[2][NW];
+  int st = 0, par = 0;          // stage of plane i and the parity of its phase
+  int zc = 0, yb = 0, yc = 0;   // component of the z pass (plane i); of the y pass (plane i - 1)
+  int xa = 0, xb = 0, xc = 0;   // components of the x pass (plane i - 2)
 #pragma unroll 1
-  for (int i = 0; i < kQ3; ++i) {
-    const int st = i & 1, ia = i / 25, ib = (i / 5) % 5, ic = i % 5;
-    const bool late = !mbar_wait(&BAR[st], (unsigned)((i >> 1) & 1), a.flag);
-    if (__syncthreads_or(late)) {   // the copy of plane i did not land in time: stop, after it
-      mbar_wait(&BAR[st], (unsigned)((i >> 1) & 1), a.flag);
+  for (int i = 0; i < kQ3 + 2; ++i) {
+    const bool late = i < kQ3 && !mbar_wait(&BAR[st], (unsigned)par, a.flag);
+    if (__syncthreads_or(late)) {
+      // the copy of plane i did not land in time: stop, after it and the ones issued behind it
+      for (int k = i, s2 = st, p2 = par; k < i + NS - 1 && k < kQ3; ++k) {
+        if (!mbar_wait(&BAR[s2], (unsigned)p2, a.flag)) break;
+        if (++s2 == NS) {
+          s2 = 0;
+          p2 ^= 1;
+        }
+      }
       return;
     }
-    if (tid == 0 && i + 1 < kQ3) issue(i + 1, st ^ 1);   // every thread is past plane i - 1
-    if (ic == 0 && ib == 0) {   // a new x component: this lane's x tail sums
+    if (tid == 0 && i + NS - 1 < kQ3) issue(i + NS - 1, st == 0 ? NS - 1 : st - 1);   // every thread is past plane i - 1
+    // z pass of plane i: column (ry, rx) of the region, the tile's z rows
+    if (i < kQ3) {
+      constexpr int ZR = (SH::ZT + NT - 1) / NT;
+      const float2* Sst = reinterpret_cast<const float2*>(base + (size_t)st * SH::kStride);
+      float2* zout = Zb + (i & 1) * SH::ZB;
+      float wz[TZ * NW];
 #pragma unroll
-      for (int q = 0; q < NW; ++q) wx[q] = Wx[(ia * kT3X + lane) * NW + q];
-    }
-    const float2* Sst = S + (size_t)st * RE;
-    // z pass: column (ry, rx) of the region, the tile's z rows
-    {
-      // the plane's z tail sums in registers; a thread's (up to) ZR columns with all loads in flight
-      constexpr int ZR = (SH::ZT + kT3NT - 1) / kT3NT;
-      float wz[kT3Z * NW];
-#pragma unroll
-      for (int q = 0; q < kT3Z * NW; ++q) wz[q] = Wz[ic * kT3Z * NW + q];
-      float2 v[ZR][RZ];
+      for (int q = 0; q < TZ * NW; ++q) wz[q] = Wz[zc * TZ * NW + q];
 #pragma unroll
       for (int c = 0; c < ZR; ++c) {
-        const int t = tid + c * kT3NT;
+        const int t = tid + c * NT;
         if (t < SH::ZT) {
+          float2 v[RZ], d[RZ - 1];
 #pragma unroll
-          for (int r = 0; r < RZ; ++r) v[c][r] = Sst[r * RY * RX + t];
+          for (int r = 0; r < RZ; ++r) v[r] = Sst[r * RY * RX + t];
+#pragma unroll
+          for (int r = 0; r + 1 < RZ; ++r) d[r] = sub2(v[r + 1], v[r]);
+#pragma unroll
+          for (int tz = 0; tz < TZ; ++tz) zout[tz * SH::ZS + t] = tail_interp<P>(v, d, tz + P, wz + tz * NW);
         }
       }
+      if (++st == NS) {
+        st = 0;
+        par ^= 1;
+      }
+      if (++zc == kQ1) zc = 0;
+    }
+    // y pass of plane i - 1: column (tz, rx), the tile's y rows
+    if (i >= 1 && i <= kQ3) {
+      if (yt >= 0) {
+        const float* wy = Wy + yb * kT3Y * NW;
+        const float2* zin = Zb + ((i - 1) & 1) * SH::ZB + ytz * SH::ZS + ycol;
+        float2* yout = Yb + ((i - 1) & 1) * SH::YB + ytz * SH::YS + ycol;
+        float2 v[RY], d[RY - 1];
 #pragma unroll
-      for (int c = 0; c < ZR; ++c) {
-        const int t = tid + c * kT3NT;
-        if (t < SH::ZT) {
-          float2 d[RZ - 1];
+        for (int r = 0; r < RY; ++r) v[r] = zin[r * RX];
 #pragma unroll
-          for (int r = 0; r + 1 < RZ; ++r) d[r] = sub2(v[c][r + 1], v[c][r]);
+        for (int r = 0; r + 1 < RY; ++r) d[r] = sub2(v[r + 1], v[r]);
 #pragma unroll
-          for (int tz = 0; tz < kT3Z; ++tz) Zb[tz * RY * RX + t] = tail_interp<P>(v[c], d, tz + P, wz + tz * NW);
-        }
+        for (int ty = 0; ty < kT3Y; ++ty) yout[ty * RX] = tail_interp<P>(v, d, ty + P, wy + ty * NW);
+      }
+      if (++yc == kQ1) {
+        yc = 0;
+        if (++yb == kQ1) yb = 0;
       }
     }
-    __syncthreads();
-    // y pass: column (tz, rx), the tile's y rows
-    if (tid < SH::YT) {
-      const int tz = tid / RX, rx = tid - tz * RX;
-      const float* wy = Wy + ib * kT3Y * NW;
-      float2 v[RY], d[RY - 1];
+    // x pass of plane i - 2: two neighbouring vertices a task, into the destination; their moments
+    if (i >= 2) {
+      if (xb == 0 && xc == 0) {   // a new x component: the tail sums of this thread's columns
 #pragma unroll
-      for (int r = 0; r < RY; ++r) v[r] = Zb[(tz * RY + r) * RX + rx];
+        for (int q = 0; q < NW; ++q) {
+          wx[0][q] = Wx[(xa * kT3X + 2 * xp) * NW + q];
+          wx[1][q] = Wx[(xa * kT3X + 2 * xp + 1) * NW + q];
+        }
+      }
+      const float ey = a.cs.xif[xb], ez = a.cs.xif[xc], e2 = ey * ey + ez * ez;
 #pragma unroll
-      for (int r = 0; r + 1 < RY; ++r) d[r] = sub2(v[r + 1], v[r]);
+      for (int k = 0; k < XT; ++k) {
+        const int row = (tid + k * NT) >> 4;
+        const float4* in = reinterpret_cast<const float4*>(Yb + (i & 1) * SH::YB + (row / kT3Y) * SH::YS +
+                                                           (row % kT3Y) * RX + 2 * xp);
+        float2 v[2 * XO + 2], d[2 * XO + 1];
 #pragma unroll
-      for (int ty = 0; ty < kT3Y; ++ty) Yb[(tz * kT3Y + ty) * RX + rx] = tail_interp<P>(v, d, ty + P, wy + ty * NW);
-    }
-    __syncthreads();
-    // x pass: the vertex (x0 + lane, row) into the destination; its moments
-    const float ex = a.cs.xif[ia], ey = a.cs.xif[ib], ez = a.cs.xif[ic];
-    const float e2 = ex * ex + ey * ey + ez * ez;
+        for (int j = 0; j <= XO; ++j) {
+          const float4 q = in[j];
+          v[2 * j] = make_float2(q.x, q.y);
+          v[2 * j + 1] = make_float2(q.z, q.w);
+        }
 #pragma unroll
-    for (int j = 0; j < XR; ++j) {
-      const int r = XR * warp + j, tz = r / kT3Y, ty = r - tz * kT3Y;
-      const float2* row = Yb + (tz * kT3Y + ty) * RX + kT3XO + lane;
-      float2 v[2 * P + 1], d[2 * P];
+        for (int j = 0; j < 2 * XO + 1; ++j) d[j] = sub2(v[j + 1], v[j]);
+        const float2 r0 = tail_interp<P>(v, d, XO, wx[0]), r1 = tail_interp<P>(v, d, XO + 1, wx[1]);
+        if (on[k]) {
+          if (both)
+            *reinterpret_cast<float4*>(out[k]) = make_float4(r0.x, r0.y, r1.x, r1.y);
+          else
+            *out[k] = r0;
+        }
+        out[k] += a.lay.plane;
+        const float2 r[2] = {r0, r1};
 #pragma unroll
-      for (int k = 0; k <= 2 * P; ++k) v[k] = row[k - P];
+        for (int v2 = 0; v2 < 2; ++v2) {
+          part[k][v2] = __fadd2_rn(part[k][v2], r[v2]);
+          my[k][v2] = fmaf(ey, r[v2].x, my[k][v2]);
+          mz[k][v2] = fmaf(ez, r[v2].x, mz[k][v2]);
+          m2[k][v2] = fmaf(e2, r[v2].x, m2[k][v2]);
+        }
+      }
+      if (++xc == kQ1) {
+        xc = 0;
+        if (++xb == kQ1) {   // the planes of one x component are done
+          xb = 0;
+          const float ex = a.cs.xif[xa];
 #pragma unroll
-      for (int k = 0; k < 2 * P; ++k) d[k] = sub2(v[k + 1], v[k]);
-      const float2 acc = tail_interp<P>(v, d, P, wx);
-      const int vy = y0 + ty, vz = z0 + tz;
-      if (vx < a.nx && vy < a.ny && vz < a.nz) {
-        a.dst[a.lay.at(i, vx, vy, vz)] = acc;
-        m[j][0] += acc.x;
-        m[j][1] += ex * acc.x;
-        m[j][2] += ey * acc.x;
-        m[j][3] += ez * acc.x;
-        m[j][4] += e2 * acc.x;
-        m[j][5] += acc.y;
+          for (int k = 0; k < XT; ++k)
+#pragma unroll
+            for (int v2 = 0; v2 < 2; ++v2) {
+              fg[k][v2] = __fadd2_rn(fg[k][v2], part[k][v2]);
+              mx[k][v2] = fmaf(ex, part[k][v2].x, mx[k][v2]);
+              m2[k][v2] = fmaf(ex * ex, part[k][v2].x, m2[k][v2]);
+              part[k][v2] = make_float2(0.f, 0.f);
+            }
+          ++xa;
+        }
       }
     }
   }
 #pragma unroll
-  for (int j = 0; j < XR; ++j) {
-    const int r = XR * warp + j, tz = r / kT3Y, ty = r - tz * kT3Y;
-    const int vy = y0 + ty, vz = z0 + tz;
-    if (vx < a.nx && vy < a.ny && vz < a.nz) {
-      const size_t v = ((size_t)vz * a.ny + vy) * a.nx + vx;
+  for (int k = 0; k < XT; ++k) {
+    const int row = (tid + k * NT) >> 4, vy = y0 + row % kT3Y, vz = z0 + row / kT3Y;
+    if (!on[k]) continue;
+    const size_t v = ((size_t)vz * a.ny + vy) * a.nx + vx;
 #pragma unroll
-      for (int q = 0; q < 6; ++q) a.sums[(size_t)q * a.nv + v] = m[j][q];
+    for (int v2 = 0; v2 < 2; ++v2) {
+      if (v2 == 1 && !both) continue;
+      const float m[6] = {fg[k][v2].x, mx[k][v2], my[k][v2], mz[k][v2], m2[k][v2], fg[k][v2].y};
+#pragma unroll
+      for (int q = 0; q < 6; ++q) a.sums[(size_t)q * a.nv + v + v2] = m[q];
     }
   }
 }
 
 // Second sweep of the sum-factorised step: one thread per vertex relaxes its 125 pairs in place
-// (read back from the destination, a row of 5 ahead), from the moment sums of the stream
-// kernel, with the residual correction of step3d_f32_kernel.  ghost_refresh3d_kernel then copies
-// the periodic images into the ghost cells.
+// (read back from the destination), from the moment sums of the stream kernel, with the residual
+// correction of step3d_f32_kernel, and writes them to the periodic images of the vertex in the
+// ghost cells as well.  It moves 16 bytes an update, at 4.9 TB/s on 128^3 vertices (0.919 ms, with
+// rows of 5 pairs asked for two rows ahead in five blocks an SM; one row ahead in six: 1.011 ms; the
+// copying of the images was a launch of 0.18 ms of its own).  Per row (a, b) the products
+// X_k(a) Y_l(b) are summed by order first, so that a velocity takes 5 multiply-adds.
 struct Collide3Args {
   float2* dst;
   Pad3 lay;
@@ -584,12 +671,49 @@ struct Collide3Args {
   int* flag;
 };
 
-__global__ void __launch_bounds__(128, 6) collide3d_kernel(const __grid_constant__ Collide3Args a) {
-  const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= a.nv) return;
-  const int x = (int)(v % a.nx), y = (int)((v / a.nx) % a.ny), z = (int)(v / ((long long)a.nx * a.ny));
-  const size_t plane = a.lay.plane;
-  float2* own = a.dst + a.lay.at(0, x, y, z);
+__global__ void __launch_bounds__(128, 5) collide3d_kernel(const __grid_constant__ Collide3Args a) {
+  const unsigned v = blockIdx.x * 128u + threadIdx.x;   // at most 2^27 vertices
+  if (v >= (unsigned)a.nv) return;
+  const unsigned yz = v / (unsigned)a.nx;
+  const int x = (int)(v - yz * (unsigned)a.nx), z = (int)(yz / (unsigned)a.ny), y = (int)(yz - (unsigned)z * (unsigned)a.ny);
+  // value i of this vertex: the plane's address (the same for all threads) and the vertex's offset
+  // in a plane
+  char* const base = reinterpret_cast<char*>(a.dst);
+  const size_t plane = a.lay.plane * sizeof(float2);
+  const size_t off = a.lay.at(0, x, y, z) * sizeof(float2);
+  auto at = [&](int i) { return reinterpret_cast<float2*>(base + (size_t)i * plane + off); };
+  // the vertex's periodic images in the ghost cells (axes are at least two ghost widths long: one
+  // image an axis).  The x image is one predicated store, since half the warps hold some; the others
+  // are whole rows and slices, behind a branch that few warps take.
+  const int g = a.lay.g;
+  const int dx = !a.px ? 0 : x < g ? a.nx : x >= a.nx - g ? -a.nx : 0;
+  const int dy = !a.py ? 0 : y < g ? a.ny : y >= a.ny - g ? -a.ny : 0;
+  const int dz = !a.pz ? 0 : z < g ? a.nz : z >= a.nz - g ? -a.nz : 0;
+  const int sy = a.lay.pitch * dy, sz = a.lay.pitch * a.lay.rows * dz;   // below a plane: < 2^31 pairs
+  auto put = [&](int i, float2 val) {
+    float2* o = at(i);
+    *o = val;
+    if (dx) o[dx] = val;
+    if (dy | dz) {
+      if (dy) {
+        o[sy] = val;
+        if (dx) o[sy + dx] = val;
+      }
+      if (dz) {
+        o[sz] = val;
+        if (dx) o[sz + dx] = val;
+        if (dy) {
+          o[sz + sy] = val;
+          if (dx) o[sz + sy + dx] = val;
+        }
+      }
+    }
+  };
+  float2 cur[kQ1], nxt[kQ1];
+#pragma unroll
+  for (int ic = 0; ic < kQ1; ++ic) cur[ic] = *at(ic);
+#pragma unroll
+  for (int ic = 0; ic < kQ1; ++ic) nxt[ic] = *at(kQ1 + ic);
   const size_t sp = (size_t)a.nv;
   const float drho = a.sums[v], jx = a.sums[sp + v], jy = a.sums[2 * sp + v], jz = a.sums[3 * sp + v],
               a2 = a.sums[4 * sp + v];
@@ -612,120 +736,135 @@ __global__ void __launch_bounds__(128, 6) collide3d_kernel(const __grid_constant
       A3[d][4] = u * u * (u * u + 6.f * q) + 3.f * q * q;
     }
   }
-  float Zc[5][5];   // [n][c]: sum_{m <= n} A_m(u_z) he_m(c)
+  // Zc[n][c] = sum_{1 <= m <= n} A_m(u_z) he_m(c): the sums to order n without their leading 1
+  float Zc[5][5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     float acc = 0.f;
+    Zc[0][c] = 0.f;
 #pragma unroll
-    for (int m = 0; m < 5; ++m) {
+    for (int m = 1; m < 5; ++m) {
       acc += Az[m] * a.cs.hef[m][c];
       Zc[m][c] = acc;
     }
   }
   const float om = a.omega, Kq1 = a.K * (1.f + q), Kq = a.K * q;
   const float2 om2 = bcast2(om);
-  float r0 = 0.f, r1 = 0.f, r2 = 0.f, r3 = 0.f, re = 0.f;
-  // rows (a, b) of 5 pairs (c = 0..4), the next row's loads in flight while one row relaxes
-  float2 cur[kQ1];
-#pragma unroll
-  for (int ic = 0; ic < kQ1; ++ic) cur[ic] = own[(size_t)ic * plane];
+  const bool two = a.npop == 2;
+  float r0 = 0.f, r1 = 0.f, r2 = 0.f, r3 = 0.f, re = 0.f, rg = 0.f;
 #pragma unroll 1
   for (int row = 0; row < kQ1 * kQ1; ++row) {
     const int ia = row / kQ1, ib = row - kQ1 * ia;
-    float2 nxt[kQ1];
-    if (row + 1 < kQ1 * kQ1) {
+    float2 aft[kQ1];   // two rows ahead
+    if (row + 2 < kQ1 * kQ1) {
 #pragma unroll
-      for (int ic = 0; ic < kQ1; ++ic) nxt[ic] = own[(size_t)(kQ1 * (row + 1) + ic) * plane];
+      for (int ic = 0; ic < kQ1; ++ic) aft[ic] = *at(kQ1 * (row + 2) + ic);
     }
-    float Xa[5], Yb[5];
+    // C[n] = sum_{k + l = 4 - n} X_k(a) Y_l(b): E - 1 = sum_n C[n] (1 + Zc[n][c]) - 1, C[4] = 1
+    float X[5], Y[5], C[4];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      Xa[k] = Ax[k] * a.cs.hef[k][ia];
-      Yb[k] = Ay[k] * a.cs.hef[k][ib];
+    for (int k = 1; k < 5; ++k) {
+      X[k] = Ax[k] * a.cs.hef[k][ia];
+      Y[k] = Ay[k] * a.cs.hef[k][ib];
     }
+    C[3] = X[1] + Y[1];
+    C[2] = X[2] + Y[2] + X[1] * Y[1];
+    C[1] = X[3] + Y[3] + X[2] * Y[1] + X[1] * Y[2];
+    C[0] = X[4] + Y[4] + X[3] * Y[1] + X[1] * Y[3] + X[2] * Y[2];
+    const float Cs = C[0] + C[1] + C[2] + C[3];
     const float ex = a.cs.xif[ia], ey = a.cs.xif[ib], wab = a.cs.wf[ia] * a.cs.wf[ib];
-    float2* o5 = own + (size_t)(kQ1 * row) * plane;
+    float rs = 0.f, rz = 0.f, rzz = 0.f;
 #pragma unroll
     for (int ic = 0; ic < kQ1; ++ic) {
-      float s1 = 0.f;
+      float em1 = Cs + Zc[4][ic];
 #pragma unroll
-      for (int k = 0; k <= 4; ++k) {
-        float sl = 0.f;
-#pragma unroll
-        for (int l = 0; l <= 4 - k; ++l) sl += Yb[l] * Zc[4 - k - l][ic];
-        s1 += Xa[k] * sl;
-      }
+      for (int n = 1; n < 4; ++n) em1 = fmaf(C[n], Zc[n][ic], em1);
       const float w = wab * a.cs.wf[ic];
-      const float ef = w * (drho + rho * (s1 - 1.f));
-      const float eg = Kq1 * ef + Kq * w;
-      const float2 d = sub2(make_float2(ef, a.npop == 2 ? eg : 0.f), cur[ic]);
+      const float ef = w * fmaf(rho, em1, drho);
+      const float eg = Kq1 * ef + Kq * w;   // g^eq - K w = K ((1 + q)(f^eq - w) + q w)
+      const float2 d = sub2(make_float2(ef, two ? eg : 0.f), cur[ic]);
       const float ez = a.cs.xif[ic];
-      r0 += d.x;
-      r1 += ex * d.x;
-      r2 += ey * d.x;
-      r3 += ez * d.x;
-      re += (ex * ex + ey * ey + ez * ez) * d.x + d.y;
-      o5[(size_t)ic * plane] = fma2(om2, d, cur[ic]);
+      rs += d.x;
+      rz = fmaf(ez, d.x, rz);
+      rzz = fmaf(ez * ez, d.x, rzz);
+      rg += d.y;
+      const float2 val = fma2(om2, d, cur[ic]);
+      put(kQ1 * row + ic, val);
     }
-    if (row + 1 < kQ1 * kQ1) {
+    r0 += rs;
+    r1 = fmaf(ex, rs, r1);
+    r2 = fmaf(ey, rs, r2);
+    r3 += rz;
+    re += fmaf(fmaf(ex, ex, ey * ey), rs, rzz);
 #pragma unroll
-      for (int ic = 0; ic < kQ1; ++ic) cur[ic] = nxt[ic];
+    for (int ic = 0; ic < kQ1; ++ic) {
+      cur[ic] = nxt[ic];
+      nxt[ic] = aft[ic];
     }
   }
   {
     const float inv_s = a.cs.inv_xi1f, s2 = a.cs.xi1sqf;
     const float d1 = r1 * inv_s, d2 = r2 * inv_s, d3 = r3 * inv_s;
     const float d0 = r0 - d1 - d2 - d3;
-    const float de = re - s2 * (d1 + d2 + d3);
-    own[0].x -= om * d0;
-    own[25 * plane].x -= om * d1;
-    own[5 * plane].x -= om * d2;
-    own[1 * plane].x -= om * d3;
-    if (a.npop == 2) {
-      own[0].y -= om * de;
-    } else if (!a.iso) {
+    const float de = re + rg - s2 * (d1 + d2 + d3);
+    // (held in registers to the end instead, these cost the fifth block: 0.956 ms against 0.919 on 128^3)
+    float2 v0 = *at(0), v1 = *at(1), v5 = *at(5), v25 = *at(25), v75 = *at(75);
+    v0.x -= om * d0;
+    v25.x -= om * d1;
+    v5.x -= om * d2;
+    v1.x -= om * d3;
+    if (two) {
+      v0.y -= om * de;
+    } else if (!a.iso) {   // one population: energy along (+-s, 0, 0) and -2 at rest
       const float e = om * 0.5f * de * inv_s * inv_s;
-      own[25 * plane].x -= e;
-      own[75 * plane].x -= e;
-      own[0].x += 2.f * e;
+      v25.x -= e;
+      v75.x -= e;
+      v0.x += 2.f * e;
     }
+    put(0, v0);
+    put(1, v1);
+    put(5, v5);
+    put(25, v25);
+    put(75, v75);
   }
   if (!((rho > 0.f) && (qk > -1.f) && isfinite(rho) && isfinite(qk))) atomicOr(a.flag, 1);
 }
 
-// The periodic images of the ghost cells of a padded pair state, one thread per (plane, ghost
-// cell).  The ghost cells of a plane are enumerated as three disjoint sets: the 2g slices before
-// and after the interior slices (whole rows), then in the interior slices the 2g ghost rows,
-// then in the interior rows the 2g ghost columns.  A cell past a zero-gradient face is skipped.
+// The periodic images of the ghost cells of a padded pair state (after init and set_state), one
+// thread per (plane, ghost cell).  The ghost cells of a plane are enumerated as three disjoint
+// sets: the 2g slices before and after the interior slices (whole rows), then in the interior
+// slices the 2g ghost rows, then in the interior rows the columns outside the interior.  A cell
+// past a zero-gradient face, or in the row padding past the ghost columns, is skipped.
 __global__ void __launch_bounds__(256) ghost_refresh3d_kernel(float2* pairs, Pad3 lay, int nx, int ny, int nz,
-                                                              int px, int py, int pz, long long per_plane) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)kQ3 * per_plane) return;
-  const int i = (int)(e / per_plane);
-  long long r = e - (long long)i * per_plane;
-  const int g = lay.g, W = lay.pitch, R = lay.rows;
-  const long long nzs = 2LL * g * R * W, nys = (long long)nz * 2 * g * W;
+                                                              int px, int py, int pz, unsigned per_plane) {
+  const unsigned e = blockIdx.x * 256u + threadIdx.x;
+  if (e >= per_plane) return;
+  const int i = blockIdx.y;
+  unsigned r = e;
+  const unsigned g = lay.g, W = lay.pitch, R = lay.rows, S = W - nx;   // S: columns outside the interior
+  const unsigned nzs = 2 * g * R * W, nys = (unsigned)nz * 2 * g * W;
   int X, Y, Z;   // interior coordinates of the ghost cell (outside [0, n) on some axis)
   if (r < nzs) {
-    const int zz = (int)(r / ((long long)R * W));
-    r -= (long long)zz * R * W;
-    Z = zz < g ? zz - g : nz + zz - g;
-    Y = (int)(r / W) - g;
-    X = (int)(r % W) - g;
+    const int zz = (int)(r / (R * W));
+    r -= (unsigned)zz * R * W;
+    Z = zz < (int)g ? zz - (int)g : nz + zz - (int)g;
+    Y = (int)(r / W) - (int)g;
+    X = (int)(r % W) - (int)g;
   } else if ((r -= nzs) < nys) {
-    Z = (int)(r / (2LL * g * W));
-    r -= (long long)Z * 2 * g * W;
+    Z = (int)(r / (2 * g * W));
+    r -= (unsigned)Z * 2 * g * W;
     const int yy = (int)(r / W);
-    Y = yy < g ? yy - g : ny + yy - g;
-    X = (int)(r % W) - g;
+    Y = yy < (int)g ? yy - (int)g : ny + yy - (int)g;
+    X = (int)(r % W) - (int)g;
   } else {
     r -= nys;
-    Z = (int)(r / ((long long)ny * 2 * g));
-    r -= (long long)Z * ny * 2 * g;
-    Y = (int)(r / (2 * g));
-    const int xx = (int)(r % (2 * g));
-    X = xx < g ? xx - g : nx + xx - g;
+    Z = (int)(r / ((unsigned)ny * S));
+    r -= (unsigned)Z * ny * S;
+    Y = (int)(r / S);
+    const int xx = (int)(r % S);
+    X = xx < (int)g ? xx - (int)g : nx + xx - (int)g;
   }
+  if (X >= nx + (int)g) return;   // row padding
   const bool ox = X < 0 || X >= nx, oy = Y < 0 || Y >= ny, oz = Z < 0 || Z >= nz;
   if ((ox && !px) || (oy && !py) || (oz && !pz)) return;
   const int x = ox ? (X < 0 ? X + nx : X - nx) : X, y = oy ? (Y < 0 ? Y + ny : Y - ny) : Y,
@@ -736,7 +875,7 @@ __global__ void __launch_bounds__(256) ghost_refresh3d_kernel(float2* pairs, Pad
 // Tail sums T+_j, -T-_j (j = 1..p) of every (component, node) of one axis, from the FP64 tables:
 // the stencil of node n starts at n + off and has weights w_0..w_p, offsets d = off + k.
 template <int P>
-__global__ void tail_table_kernel(const int* off, const double* w, int n, float* out) {
+__global__ void __launch_bounds__(128) tail_table_kernel(const int* off, const double* w, int n, float* out) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= kQ1 * n) return;
   double W[2 * P + 1];
@@ -744,7 +883,8 @@ __global__ void tail_table_kernel(const int* off, const double* w, int n, float*
   for (int d = 0; d <= 2 * P; ++d) W[d] = 0.0;
   const int o = off[e];
 #pragma unroll
-  for (int k = 0; k <= P; ++k) W[o + k + P] += w[(size_t)e * (P + 1) + k];   // o + k in [-P, P]
+  for (int k = 0; k <= P; ++k)   // o + k is in [-P, P] (tiled3d_usable)
+    if (o + k >= -P && o + k <= P) W[o + k + P] += w[(size_t)e * (P + 1) + k];
 #pragma unroll
   for (int j = 1; j <= P; ++j) {
     double tp = 0.0, tm = 0.0;
@@ -755,45 +895,51 @@ __global__ void tail_table_kernel(const int* off, const double* w, int n, float*
   }
 }
 
-// FP32 pairs (layout lay) <-> dense FP64 full populations [npop][125][nv].
-__global__ void convert3d_kernel(float2* pairs, Pad3 lay, double* dense, int nx, int ny, long long nv, int npop,
-                                 double K, Consts cs, int to_dense) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)kQ3 * nv) return;
-  const int i = (int)(e / nv);
-  const long long v = e - (long long)i * nv;
-  const int x = (int)(v % nx), y = (int)((v / nx) % ny), z = (int)(v / ((long long)nx * ny));
-  const size_t o = lay.at(i, x, y, z);
-  const double w = cs.w[i / 25] * cs.w[(i / 5) % 5] * cs.w[i % 5];
-  if (to_dense) {
-    const float2 p = pairs[o];
-    dense[e] = (double)p.x + w;
-    if (npop == 2) dense[(size_t)kQ3 * nv + e] = (double)p.y + K * w;
-  } else {
-    const float f = (float)(dense[e] - w);
-    const float g = npop == 2 ? (float)(dense[(size_t)kQ3 * nv + e] - K * w) : 0.f;
-    pairs[o] = make_float2(f, g);
+// FP32 pairs (layout lay) <-> dense FP64 full populations [npop][125][nv]: plane i = blockIdx.y, whose
+// lattice weights the block forms once.  (With four FP64 products a value and FP64 conversions the
+// FP64 pipe bound it: 2.94 ms for the 2.1 M vertices of 128^3, now 1.37 ms, 0.95 ms of it HBM traffic.)
+constexpr int kConvPer = 4;   // vertices a thread
+__global__ void __launch_bounds__(256) convert3d_kernel(float2* pairs, Pad3 lay, double* dense, int nx, int ny,
+                                                        unsigned nv, int npop, double K, const __grid_constant__ Consts cs,
+                                                        int to_dense) {
+  __shared__ double ws[2];
+  const int i = blockIdx.y;
+  if (threadIdx.x == 0) {
+    ws[0] = cs.w[i / 25] * cs.w[(i / 5) % 5] * cs.w[i % 5];
+    ws[1] = K * ws[0];
   }
-}
-
-// Periodic images of a ghost-padded pair state: every ghost cell whose position lies past
-// periodic faces only takes the value of the interior vertex it images (ghosts past a
-// zero-gradient face stay as they are: zero, never read by an interior vertex).
-__global__ void ghost3d_kernel(float2* pairs, Pad3 lay, int nx, int ny, int nz, int px, int py, int pz) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int slices = nz + 2 * lay.g;
-  const long long per_plane = (long long)lay.pitch * lay.rows * slices;
-  if (e >= (long long)kQ3 * per_plane) return;
-  const int i = (int)(e / per_plane);
-  const long long r = e - (long long)i * per_plane;
-  const int X = (int)(r % lay.pitch) - lay.g, Y = (int)((r / lay.pitch) % lay.rows) - lay.g,
-            Z = (int)(r / ((long long)lay.pitch * lay.rows)) - lay.g;
-  const bool ox = X < 0 || X >= nx, oy = Y < 0 || Y >= ny, oz = Z < 0 || Z >= nz;
-  if (!(ox || oy || oz) || X >= nx + lay.g) return;   // interior, or row padding past the ghosts
-  if ((ox && !px) || (oy && !py) || (oz && !pz)) return;
-  const int x = ox ? (X < 0 ? X + nx : X - nx) : X, y = oy ? (Y < 0 ? Y + ny : Y - ny) : Y,
-            z = oz ? (Z < 0 ? Z + nz : Z - nz) : Z;
-  pairs[(size_t)i * lay.plane + r] = pairs[lay.at(i, x, y, z)];
+  __syncthreads();
+  const double w = ws[0], Kw = ws[1];
+  double *df = dense + (size_t)i * nv, *dg = dense + (size_t)(kQ3 + i) * nv;
+  unsigned v[kConvPer];
+  size_t o[kConvPer];
+#pragma unroll
+  for (int k = 0; k < kConvPer; ++k) {
+    v[k] = (blockIdx.x * kConvPer + k) * 256u + threadIdx.x;
+    const unsigned vk = min(v[k], nv - 1), yz = vk / (unsigned)nx, z = yz / (unsigned)ny;
+    o[k] = lay.at(i, (int)(vk - yz * (unsigned)nx), (int)(yz - z * (unsigned)ny), (int)z);
+  }
+  if (to_dense) {
+    float2 p[kConvPer];
+#pragma unroll
+    for (int k = 0; k < kConvPer; ++k) p[k] = pairs[o[k]];   // past the end: the last vertex again
+#pragma unroll
+    for (int k = 0; k < kConvPer; ++k)
+      if (v[k] < nv) {
+        df[v[k]] = exact_double(p[k].x) + w;
+        if (npop == 2) dg[v[k]] = exact_double(p[k].y) + Kw;
+      }
+  } else {
+    double f[kConvPer], g[kConvPer];
+#pragma unroll
+    for (int k = 0; k < kConvPer; ++k) {
+      f[k] = df[min(v[k], nv - 1)];
+      g[k] = npop == 2 ? dg[min(v[k], nv - 1)] : Kw;
+    }
+#pragma unroll
+    for (int k = 0; k < kConvPer; ++k)
+      if (v[k] < nv) pairs[o[k]] = make_float2(nearest_float(f[k] - w), nearest_float(g[k] - Kw));
+  }
 }
 
 __global__ void init3d_kernel(const __grid_constant__ Field3Args a) {
@@ -926,7 +1072,7 @@ struct sllbm3d_ctx {
   int* off[3] = {nullptr, nullptr, nullptr};
   float* w32[3] = {nullptr, nullptr, nullptr};
   double* w64[3] = {nullptr, nullptr, nullptr};
-  // sum-factorised FP32 step (orders 1, 2 with an even x count): tail sums per axis, moment sums
+  // sum-factorised FP32 step: tail sums per axis, moment sums
   bool tiled = false;
   Pad3 lay{};                            // layout of the FP32 pair state
   float* tail[3] = {nullptr, nullptr, nullptr};
@@ -975,6 +1121,7 @@ cudaError_t launch_stream3d(const Stream3Args& a, cudaStream_t s) {
   using SH = T3Shape<P>;
   EncodeTiledFn enc = encode_fn();
   if (!enc) return cudaErrorNotSupported;
+  if (a.lay.g != SH::G || a.lay.pitch % 2) return cudaErrorInvalidValue;
   // 4D map of the ghost-padded source pairs as floats: (2 x column, row, slice, velocity plane)
   CUtensorMap smap;
   const cuuint64_t dims[4] = {(cuuint64_t)2 * a.lay.pitch, (cuuint64_t)a.lay.rows,
@@ -990,17 +1137,38 @@ cudaError_t launch_stream3d(const Stream3Args& a, cudaStream_t s) {
     return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(stream3d_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::kBytes);
   if (e != cudaSuccess) return e;
-  const long long tiles = (long long)((a.nx + kT3X - 1) / kT3X) * ((a.ny + kT3Y - 1) / kT3Y) * ((a.nz + kT3Z - 1) / kT3Z);
-  stream3d_kernel<P><<<(unsigned)tiles, kT3NT, SH::kBytes, s>>>(a, smap);
+  const long long tiles = (long long)((a.nx + kT3X - 1) / kT3X) * ((a.ny + kT3Y - 1) / kT3Y) * ((a.nz + SH::TZ - 1) / SH::TZ);
+  stream3d_kernel<P><<<(unsigned)tiles, SH::NT, SH::kBytes, s>>>(a, smap);
   return cudaGetLastError();
+}
+
+// Whether the sum-factorised step takes the grid: FP32, axes at least as long as a staged region of
+// order 2 (36 x 12 x 8 vertices; also two ghost widths), and every stencil within p vertices of its vertex: from
+// an inner node the departures stay in the cell, from a cell face they reach no further than the
+// neighbouring cells.
+bool tiled3d_usable(const sllbm3d_ctx* c, double dt) {
+  if (!c->f32 || encode_fn() == nullptr) return false;
+  const AxisK* axes[3] = {&c->ax, &c->ay, &c->az};
+  const int least[3] = {36, 12, 8};
+  for (int k = 0; k < 3; ++k) {
+    const AxisK& ax = *axes[k];
+    if (ax.nv < least[k] || (ax.periodic && ax.n_cells < 3)) return false;   // (two cells: each is both neighbours)
+    for (int a = 0; a < kQ1; ++a) {
+      const double d = dt * c->cs.xi[a] / ax.hc;   // in cells; 1e-9 keeps clear of rounding
+      if (!(fabs(d) < 1.0 - 1e-9)) return false;
+      for (int l = 1; l < ax.p; ++l)
+        if (!(ax.nodes[l] - d > 1e-9 && ax.nodes[l] - d < 1.0 - 1e-9)) return false;
+    }
+  }
+  return true;
 }
 
 // The periodic images of the current state's ghost cells (after init and set_state).
 cudaError_t fill_ghosts3d(sllbm3d_ctx* c) {
   if (!c->tiled) return cudaSuccess;
-  const long long n = (long long)kQ3 * (long long)c->lay.plane;
-  ghost3d_kernel<<<blocks_for(n, 256), 256, 0, c->stream>>>(pairs(c, c->cur), c->lay, c->ax.nv, c->ay.nv, c->az.nv,
-                                                           c->ax.periodic, c->ay.periodic, c->az.periodic);
+  const unsigned per_plane = (unsigned)(c->lay.plane - (size_t)c->nv);   // cells outside the interior
+  ghost_refresh3d_kernel<<<dim3((per_plane + 255) / 256, kQ3), 256, 0, c->stream>>>(
+      pairs(c, c->cur), c->lay, c->ax.nv, c->ay.nv, c->az.nv, c->ax.periodic, c->ay.periodic, c->az.periodic, per_plane);
   return cudaGetLastError();
 }
 
@@ -1019,7 +1187,13 @@ cudaError_t launch_tiled3d(sllbm3d_ctx* c, const float2* src, float2* dst) {
   a.tz = c->tail[2];
   a.cs = c->cs;
   a.flag = c->flag;
-  cudaError_t e = c->g.order == 1 ? launch_stream3d<1>(a, c->stream) : launch_stream3d<2>(a, c->stream);
+  cudaError_t e = cudaErrorInvalidValue;
+  switch (c->g.order) {
+    case 1: e = launch_stream3d<1>(a, c->stream); break;
+    case 2: e = launch_stream3d<2>(a, c->stream); break;
+    case 3: e = launch_stream3d<3>(a, c->stream); break;
+    case 4: e = launch_stream3d<4>(a, c->stream); break;
+  }
   if (e != cudaSuccess) return e;
   Collide3Args b{};
   b.dst = dst;
@@ -1041,11 +1215,6 @@ cudaError_t launch_tiled3d(sllbm3d_ctx* c, const float2* src, float2* dst) {
   b.iso = c->p.isothermal;
   b.flag = c->flag;
   collide3d_kernel<<<blocks_for(c->nv, 128), 128, 0, c->stream>>>(b);
-  cudaError_t e2 = cudaGetLastError();
-  if (e2 != cudaSuccess) return e2;
-  const long long per_plane = (long long)c->lay.plane - c->nv;   // ghost cells of a plane
-  ghost_refresh3d_kernel<<<blocks_for((long long)kQ3 * per_plane, 256), 256, 0, c->stream>>>(
-      dst, c->lay, b.nx, b.ny, b.nz, b.px, b.py, b.pz, per_plane);
   return cudaGetLastError();
 }
 
@@ -1084,14 +1253,11 @@ sllbm_status sllbm3d_create(const sllbm_grid3_desc* g, const sllbm_params* p, vo
   c->nv = (long long)c->ax.nv * c->ay.nv * c->az.nv;
   c->npop = p->cv == 1.5 ? 1 : 2;
   c->f32 = p->prec == SLLBM_PREC_F32;
-  // the sum-factorised FP32 step: orders 1, 2, an even x count (16-byte pair rows), and axes at
-  // least as long as its staged region (36 x 12 x 8 vertices); its state keeps ghost cells
-  c->tiled = c->f32 && g->order <= 2 && c->ax.nv % 2 == 0 && c->ax.nv >= T3Shape<2>::RX &&
-             c->ay.nv >= T3Shape<2>::RY && c->az.nv >= T3Shape<2>::RZ && encode_fn() != nullptr;
+  c->tiled = tiled3d_usable(c, p->dt);   // its state keeps ghost cells, in rows of whole 16-byte units
   {
     Pad3& L = c->lay;
-    L.g = c->tiled ? kT3G : 0;
-    L.pitch = c->ax.nv + 2 * L.g;
+    L.g = c->tiled ? (g->order <= 2 ? T3Shape<2>::G : T3Shape<4>::G) : 0;
+    L.pitch = c->tiled ? (c->ax.nv + 2 * L.g + 1) / 2 * 2 : c->ax.nv;
     L.rows = c->ay.nv + 2 * L.g;
     L.plane = (size_t)L.pitch * L.rows * (c->az.nv + 2 * L.g);
     L.origin = ((size_t)L.g * L.rows + L.g) * L.pitch + L.g;
@@ -1156,10 +1322,13 @@ sllbm_status sllbm3d_precompute_departures(sllbm3d_ctx* c) {
         const sllbm_status s = alloc3(c, &c->tail[k], (size_t)kQ1 * n * 2 * P);
         if (s != SLLBM_OK) return s;
       }
-      if (P == 1)
-        tail_table_kernel<1><<<blocks_for((long long)kQ1 * n, 128), 128, 0, c->stream>>>(c->off[k], c->w64[k], n, c->tail[k]);
-      else
-        tail_table_kernel<2><<<blocks_for((long long)kQ1 * n, 128), 128, 0, c->stream>>>(c->off[k], c->w64[k], n, c->tail[k]);
+      const unsigned nb = blocks_for((long long)kQ1 * n, 128);
+      switch (P) {
+        case 1: tail_table_kernel<1><<<nb, 128, 0, c->stream>>>(c->off[k], c->w64[k], n, c->tail[k]); break;
+        case 2: tail_table_kernel<2><<<nb, 128, 0, c->stream>>>(c->off[k], c->w64[k], n, c->tail[k]); break;
+        case 3: tail_table_kernel<3><<<nb, 128, 0, c->stream>>>(c->off[k], c->w64[k], n, c->tail[k]); break;
+        default: tail_table_kernel<4><<<nb, 128, 0, c->stream>>>(c->off[k], c->w64[k], n, c->tail[k]); break;
+      }
       const sllbm_status s = cuda3(c, cudaGetLastError(), "tail_table_kernel");
       if (s != SLLBM_OK) return s;
     }
@@ -1323,8 +1492,8 @@ sllbm_status sllbm3d_moments(sllbm3d_ctx* c, double* rho, double* u, double* v, 
 sllbm_status sllbm3d_get_state(sllbm3d_ctx* c, double* dst) {
   if (!c || !dst) return fail3(c, SLLBM_ERR_ARG, "null pointer");
   if (c->f32) {
-    convert3d_kernel<<<blocks_for((long long)kQ3 * c->nv, 256), 256, 0, c->stream>>>(
-        pairs(c, c->cur), c->lay, dst, c->ax.nv, c->ay.nv, c->nv, c->npop, 2.0 * c->p.cv - 3.0, c->cs, 1);
+    convert3d_kernel<<<dim3(blocks_for(c->nv, 256 * kConvPer), kQ3), 256, 0, c->stream>>>(
+        pairs(c, c->cur), c->lay, dst, c->ax.nv, c->ay.nv, (unsigned)c->nv, c->npop, 2.0 * c->p.cv - 3.0, c->cs, 1);
     return cuda3(c, cudaGetLastError(), "convert3d_kernel");
   }
   return cuda3(c, cudaMemcpyAsync(dst, c->state[c->cur], state_doubles(c) * sizeof(double), cudaMemcpyDeviceToDevice,
@@ -1334,8 +1503,8 @@ sllbm_status sllbm3d_get_state(sllbm3d_ctx* c, double* dst) {
 sllbm_status sllbm3d_set_state(sllbm3d_ctx* c, const double* src) {
   if (!c || !src) return fail3(c, SLLBM_ERR_ARG, "null pointer");
   if (c->f32) {
-    convert3d_kernel<<<blocks_for((long long)kQ3 * c->nv, 256), 256, 0, c->stream>>>(
-        pairs(c, c->cur), c->lay, const_cast<double*>(src), c->ax.nv, c->ay.nv, c->nv, c->npop,
+    convert3d_kernel<<<dim3(blocks_for(c->nv, 256 * kConvPer), kQ3), 256, 0, c->stream>>>(
+        pairs(c, c->cur), c->lay, const_cast<double*>(src), c->ax.nv, c->ay.nv, (unsigned)c->nv, c->npop,
         2.0 * c->p.cv - 3.0, c->cs, 0);
     sllbm_status s = cuda3(c, cudaGetLastError(), "convert3d_kernel");
     if (s == SLLBM_OK) s = cuda3(c, fill_ghosts3d(c), "ghost3d_kernel");
