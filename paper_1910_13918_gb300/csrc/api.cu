@@ -291,14 +291,15 @@ static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const int* off_d
                                  bool is_y, AxisPattern& pat, bool* ok) {
   std::vector<unsigned char>& stdv = pat.follows;
   const int n = ax.nv, P = c->P;
-  std::vector<int> off((size_t)kQ1 * n);
-  std::vector<double> w((size_t)kQ1 * n * (P + 1));
+  const int nq1 = c->nq1;
+  std::vector<int> off((size_t)nq1 * n);
+  std::vector<double> w((size_t)nq1 * n * (P + 1));
   CUDA_TRY(c, cudaMemcpyAsync(off.data(), off_dev, off.size() * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(w.data(), w_dev, w.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   *ok = ax.n_cells >= 3;
   const int jref0 = (ax.n_cells / 2) * P;
-  for (int comp = 0; comp < kQ1 && *ok; ++comp)
+  for (int comp = 0; comp < nq1 && *ok; ++comp)
     for (int k = 0; k < P; ++k) {
       const int j = jref0 + k;
       const int d = off[(size_t)comp * n + j];
@@ -315,7 +316,7 @@ static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const int* off_d
   stdv.assign(n, 1);
   for (int j = 0; j < n && *ok; ++j) {
     const int k = j % P;
-    for (int comp = 0; comp < kQ1; ++comp) {
+    for (int comp = 0; comp < nq1; ++comp) {
       const int d = off[(size_t)comp * n + j];
       const double* wj = &w[((size_t)comp * n + j) * (P + 1)];
       const int dref = off[(size_t)comp * n + jref0 + k];
@@ -325,9 +326,9 @@ static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const int* off_d
       if (!same) stdv[j] = 0;
     }
   }
-  pat.tail.resize((size_t)kQ1 * n);
-  pat.before.resize((size_t)kQ1 * n);
-  for (int comp = 0; comp < kQ1; ++comp)
+  pat.tail.resize((size_t)nq1 * n);
+  pat.before.resize((size_t)nq1 * n);
+  for (int comp = 0; comp < nq1; ++comp)
     for (int j = 0; j < n; ++j) {
       const size_t e = (size_t)comp * n + j;
       float tail[4] = {0.f, 0.f, 0.f, 0.f};
@@ -351,7 +352,8 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c) {
   // Any vertex count: the tensor copies start on 16-byte boundaries of the padded rows whatever nx
   // is, and the ghost cells carry the periodic seam.  (Periodic axes of nx % 4 != 0 took the gather
   // kernel before: 1.13 ms a step on 1023 x 1023 vertices of order 3, 0.106 ms here.)
-  if (c->xs != 2) return SLLBM_OK;
+  const bool q9 = c->nq1 == 3;
+  if (c->xs != 2 && !(q9 && c->store != kStoreF64)) return SLLBM_OK;
   AxisPattern px, py;
   const std::vector<unsigned char>&sx = px.follows, &sy = py.follows;
   bool okx = false, oky = false;
@@ -361,12 +363,16 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c) {
   // The fused kernel takes each stencil as a whole cell, on both axes: start offset -l at local
   // node l, or -P at node 0 (a departure into the cell before).  Anything else goes to the
   // gather path.
-  for (int comp = 0; comp < kQ1; ++comp)
+  for (int comp = 0; comp < c->nq1; ++comp)
     for (int k = 0; k < c->P; ++k) {
       const int dy = c->ut.dy_pat[comp][k], dx = c->ut.dx_pat[comp][k];
       if (k == 0 ? (dy != 0 && dy != -c->P) : dy != -k) return SLLBM_OK;
       if (k == 0 ? (dx != 0 && dx != -c->P) : dx != -k) return SLLBM_OK;
     }
+  if (q9) {   // the whole-cell D2Q9 kernel: every vertex on the pattern, so periodic axes only
+    c->ut.valid = px.lo == 0 && px.hi == c->nx && py.lo == 0 && py.hi == c->ny;
+    return SLLBM_OK;
+  }
   if (!c->std_x) {
     TRY(dalloc(c, &c->std_x, (size_t)c->nx));
     TRY(dalloc(c, &c->std_y, (size_t)c->ny));
@@ -903,9 +909,11 @@ sllbm_status sllbm_precompute_departures(sllbm_ctx* c) {
   if (c->kernel == kKernelQ9 && (c->store == kStoreF32 || c->store == kStoreBF16) && !mapped) {
     StepArgs a = step_args(c, c->state[0], c->state[1]);
     a.mapped = 0;
-    c->q9_tma = q9_tma_usable(a, c->elem) ? 1 : 0;
+    TRY(build_uniform_pattern(c));
+    c->q9_tma = !c->ut.valid && q9_tma_usable(a, c->elem) ? 1 : 0;
   }
-  c->ghost.on = (c->kernel == kKernelUniform || c->kernel == kKernelMapped || c->q9_tma) &&
+  c->ghost.on = (c->kernel == kKernelUniform || c->kernel == kKernelMapped || c->q9_tma ||
+                 (c->kernel == kKernelQ9 && c->ut.valid)) &&
                 (c->ax.periodic || c->ay.periodic);
   double glx[8], glw[8];
   const int ngl = c->P + 3;
@@ -970,7 +978,7 @@ static cudaError_t enqueue_step(sllbm_ctx* c, float* mom = nullptr) {
       }
       break;
     case kKernelPlainF64: e = launch_step_plain_f64(a, c->stream); break;
-    case kKernelQ9: e = launch_step_q9(a, c->store, c->stream); break;
+    case kKernelQ9: e = launch_step_q9(a, c->ut, c->store, c->stream); break;
     default: e = launch_step_gather(a, c->store, c->stream); break;
   }
   if (e == cudaSuccess) c->cur ^= 1;

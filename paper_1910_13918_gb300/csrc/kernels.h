@@ -114,8 +114,10 @@ void uniform_edge_tiles(int P, int nx, int ny, UniformTables& t, std::vector<int
 // Plain FP64 step on full populations.
 cudaError_t launch_step_plain_f64(const StepArgs& a, cudaStream_t s);
 // D2Q9 step (isothermal, one population, planar storage): FP32 arithmetic on FP32/BF16
-// deviations or FP64 on full populations; per-axis tables or, with a.mapped, descriptors.
-cudaError_t launch_step_q9(const StepArgs& a, int store, cudaStream_t s);
+// deviations or FP64 on full populations; per-axis tables or, with a.mapped, descriptors.  With
+// t.valid (every vertex of a periodic uniform grid follows the cell pattern; the host keeps the
+// ghost images) FP32 and BF16 take the whole-cell kernel.
+cudaError_t launch_step_q9(const StepArgs& a, const UniformTables& t, int store, cudaStream_t s);
 // Whether the TMA-staged D2Q9 kernel can take this uniform grid with elem-byte storage (FP32 or
 // BF16: its window fits the shared memory and the ghost cells); the host then keeps the periodic
 // images in the ghost cells.
@@ -149,6 +151,7 @@ struct InitArgs {
   Consts cs;
   CollideK cp;
   int store;
+  double wh[kQ1][3];   // w_c he[k][c], c = 0, 1, 2 (set by the launch)
 };
 cudaError_t launch_init_equilibrium(const InitArgs& a, cudaStream_t s);
 // Dense [npop][nq][ny][nx] <-> internal layout (interior origin `internal`), element size `elem`,
@@ -180,6 +183,7 @@ struct MomentArgs {
   float *rho, *u, *v, *T;
   double* partials;   // [2][nblocks] scratch for the deterministic reduction
   double* sums;       // [2] device result (may be null when partials is null)
+  double inv2cv;      // 1 / (2 C_v) (set by the launch)
   int* flag;
 };
 int moments_blocks(long long nv);
@@ -238,6 +242,7 @@ struct InitVjpArgs {
   long long nv;
   Consts cs;
   CollideK cp;
+  double wh[kQ1][3];   // w_c he[k][c], c = 0, 1, 2 (set by the launch)
 };
 cudaError_t launch_init_vjp(const InitVjpArgs& a, cudaStream_t s);
 

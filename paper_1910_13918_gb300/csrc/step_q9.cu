@@ -7,8 +7,9 @@
 // invariance that the comparison shows).
 //
 // One population (the isothermal configuration) in planar storage, velocity i = 3a + b:
-// FP32 / BF16 deviations f_i - w_i with FP32 arithmetic, or FP64 full populations.  Uniform
-// grids in FP32 / BF16 run the tiled kernel below (shared-memory windows, sum factorisation);
+// FP32 / BF16 deviations f_i - w_i with FP32 arithmetic, or FP64 full populations.  Periodic
+// uniform grids in FP32 / BF16 run the whole-cell kernel (every stencil repeats with the cells),
+// uniform grids with zero-gradient axes the window kernels (per-vertex taps, sum factorisation);
 // transformed grids, FP64, and uniform grids whose departures reach farther than its window run
 // the gather kernel: one thread per vertex reads the (p+1)^2 stencil of each of the 9 planes
 // through L1/L2 (per-axis tables, or the per-(velocity, vertex) cells and local coordinates).
@@ -634,8 +635,330 @@ static cudaError_t launch_q9_tma(const StepArgs& a, const Window& win, Q9Tma qt,
   return cudaGetLastError();
 }
 
+// ---- periodic uniform grids whose stencils repeat with the cells: both passes over whole cells ----
+//
+// Persistent CTAs over tiles of 32 x TY vertices.  The window of the tile's 9 planes arrives by
+// three tensor copies on one mbarrier, two buffers, the next tile's copies in flight during this
+// one.  y pass: a thread takes one plane and two neighbouring staged columns (packed FP32x2
+// arithmetic), keeps their TY + p + 1 rows in registers and forms all TY results: one shared load
+// per row in place of p + 1.  Its results are stored as pairs of neighbouring rows, so that in
+// the x pass a thread takes two vertices, (x, y) and (x, y + 1), and everything up to the store,
+// the collision included, runs on packed pairs.  Components at rest (a = 0, b = 0) are copied, not
+// interpolated.  One barrier a tile: T is double-buffered.
+//
+// What bounds it: issue, as the tap-by-tap kernel below (step_q9_tma_kernel: 1005 warp
+// instructions per 32 vertices, mostly 4-byte shared loads), at a fraction of its instructions:
+// 2048 x 2048 vertices, p = 4, FP32: 77 us a step, 169 us with that kernel (302 MB, 44 us of traffic).
+template <int P>
+struct Q9Tile {
+  static constexpr int TY = P == 3 ? 12 : 16;       // a multiple of p, even
+  static constexpr int NT = 32 * TY / 2;            // one pair of vertices per thread
+  static constexpr int R = TY + P + 1;              // staged rows y0 - p .. y0 + TY
+  static constexpr int CP = (32 + 2 * ((P + 1) / 2 * 2)) / 2;   // column pairs of the y pass
+  static constexpr int TW = 2 * CP;                 // row length of T (pairs of rows)
+  static_assert(kN * CP <= NT, "one y task per thread at most");
+};
+template <typename Store>
+struct Q9Stage {
+  static constexpr int CO = 32 / (int)sizeof(Store) / 2;   // staged columns before the tile: 16 bytes
+  static constexpr int C = 32 + 2 * CO;
+};
 template <int P, typename Store>
-cudaError_t launch_ps(const StepArgs& a, cudaStream_t s) {
+constexpr int q9_cell_group() {   // elements of one copy (3 planes), 128-byte aligned
+  return (3 * Q9Tile<P>::R * Q9Stage<Store>::C * (int)sizeof(Store) + 127) / 128 * 128 / (int)sizeof(Store);
+}
+template <int P, typename Store>
+constexpr size_t q9_cell_smem() {
+  return 128 + sizeof(Store) * 2 * kQ9Groups * q9_cell_group<P, Store>() +
+         sizeof(float2) * 2 * kN * (Q9Tile<P>::TY / 2) * Q9Tile<P>::TW + sizeof(uint64_t) * 2;
+}
+
+template <int P>
+struct Q9CellArgs {
+  CUtensorMap tmap;
+  StepArgs a;
+  float wx[kN1][P][P], wy[kN1][P][P];   // tail sums W_1..W_P per (component, local node)
+  int bx[kN1], by[kN1];                 // 1: the stencil of local node 0 is the cell before
+};
+
+__device__ __forceinline__ float2 q9_lds2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ float2 q9_lds2(const __nv_bfloat16* p) {
+  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+
+// collide_q9_f32 of two vertices.  With He_3 = 0 on the nodes, per axis p = u he_1 + u^2 he_2 and
+// s = p + u^4 he_4: em1(a, b) = s_a + s_b + p_a p_b, the terms of total order up to four.
+__device__ __forceinline__ bool collide_q9_pair(float2 (&fb)[kN], const Consts& cs, const CollideK& cp) {
+  float2 row[kN1], col[kN1];
+#pragma unroll
+  for (int k = 0; k < kN1; ++k) {
+    row[k] = add2(add2(fb[kN1 * k], fb[kN1 * k + 1]), fb[kN1 * k + 2]);
+    col[k] = add2(add2(fb[k], fb[k + kN1]), fb[k + 2 * kN1]);
+  }
+  const float2 drho = add2(add2(row[0], row[1]), row[2]);
+  const float2 one = bcast2(1.f), rho = add2(one, drho);
+  const float2 inv = make_float2(__frcp_rn(rho.x), __frcp_rn(rho.y));
+  // xi = 0, +s, -s
+  const float2 s1 = bcast2(cs.xif[1]);
+  const float2 ux = mul2(mul2(s1, sub2(row[1], row[2])), inv), uy = mul2(mul2(s1, sub2(col[1], col[2])), inv);
+  float2 px[kN1], sx[kN1], py[kN1], sy[kN1];
+  const float2 ux2 = mul2(ux, ux), uy2 = mul2(uy, uy), ux4 = mul2(ux2, ux2), uy4 = mul2(uy2, uy2);
+#pragma unroll
+  for (int k = 0; k < kN1; ++k) {
+    const float2 h1 = bcast2(cs.hef[1][k]), h2 = bcast2(cs.hef[2][k]), h4 = bcast2(cs.hef[4][k]);
+    px[k] = mul2(ux2, h2);
+    py[k] = mul2(uy2, h2);
+    if (k > 0) {
+      px[k] = fma2(ux, h1, px[k]);
+      py[k] = fma2(uy, h1, py[k]);
+    }
+    sx[k] = fma2(ux4, h4, px[k]);
+    sy[k] = fma2(uy4, h4, py[k]);
+  }
+  const float2 om = bcast2(cp.omegaf);
+  float2 rr[kN1], rc[kN1];   // row and column sums of f^eq - f
+#pragma unroll
+  for (int k = 0; k < kN1; ++k) rr[k] = rc[k] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int a = 0; a < kN1; ++a)
+#pragma unroll
+    for (int b = 0; b < kN1; ++b) {
+      const int i = kN1 * a + b;
+      const float2 em1 = fma2(px[a], py[b], add2(sx[a], sy[b]));
+      const float2 ef = mul2(bcast2(cs.wf[a] * cs.wf[b]), fma2(rho, em1, drho));
+      const float2 d = sub2(ef, fb[i]);
+      rr[a] = add2(rr[a], d);
+      rc[b] = add2(rc[b], d);
+      fb[i] = fma2(om, d, fb[i]);
+    }
+  // remove om (r0 + r1 xi_x + r2 xi_y) w_i: sum w = 1, sum w xi xi = I on D2Q9
+  const float2 r0 = mul2(om, add2(add2(rr[0], rr[1]), rr[2]));
+  const float2 s2 = bcast2(cs.xif[1] * cs.xif[1]);
+  const float2 r1 = mul2(mul2(om, s2), sub2(rr[1], rr[2])), r2 = mul2(mul2(om, s2), sub2(rc[1], rc[2]));
+  const float2 ca[kN1] = {r0, add2(r0, r1), sub2(r0, r1)};
+#pragma unroll
+  for (int a = 0; a < kN1; ++a)
+#pragma unroll
+    for (int b = 0; b < kN1; ++b) {
+      const float2 c = b == 0 ? ca[a] : (b == 1 ? add2(ca[a], r2) : sub2(ca[a], r2));
+      fb[kN1 * a + b] = fma2(bcast2(-cs.wf[a] * cs.wf[b]), c, fb[kN1 * a + b]);
+    }
+  return rho.x > 0.f && rho.y > 0.f && isfinite(rho.x) && isfinite(rho.y) && isfinite(ux.x) && isfinite(ux.y) &&
+         isfinite(uy.x) && isfinite(uy.y);
+}
+
+template <int P, typename Store>
+__global__ void __launch_bounds__(Q9Tile<P>::NT, 2) step_q9_cell_kernel(const __grid_constant__ Q9CellArgs<P> qa) {
+  using QT = Q9Tile<P>;
+  using QS = Q9Stage<Store>;
+  constexpr int TY = QT::TY, R = QT::R, TW = QT::TW, C = QS::C, GE = q9_cell_group<P, Store>();
+  constexpr int C0 = QS::CO - (P + 1) / 2 * 2;   // first staged column of the y pass (even)
+  constexpr int TB = kN * (TY / 2) * TW;         // pairs of one T buffer
+  const StepArgs& a = qa.a;
+  extern __shared__ unsigned char q9c_smem[];
+  Store* S = reinterpret_cast<Store*>(q9c_smem + ((128 - (smem_u32(q9c_smem) & 127)) & 127));   // [2][3][3][R][C]
+  float2* T = reinterpret_cast<float2*>(S + 2 * kQ9Groups * GE);                                // [2][9][TY / 2][TW]
+  uint64_t* BAR = reinterpret_cast<uint64_t*>(T + 2 * TB);
+  const int tid = threadIdx.x, lane = tid & 31, rp = tid >> 5;   // x pass: column and row pair
+  const int tiles_x = (a.nx + 31) / 32, ntiles = tiles_x * ((a.ny + TY - 1) / TY);
+  if (tid == 0) {
+    mbar_init(&BAR[0], 1);
+    mbar_init(&BAR[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncthreads();
+  pdl_wait();   // the step before has written the source and is done with the destination
+  auto issue = [&](int tile, int buf) {   // thread 0
+    if (tile >= ntiles) return;
+    const int tx0 = (tile % tiles_x) * 32, ty0 = (tile / tiles_x) * TY;
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    mbar_expect_tx(&BAR[buf], (unsigned)(sizeof(Store) * kN * R * C));
+#pragma unroll
+    for (int g = 0; g < kQ9Groups; ++g)
+      tma_load_3d(S + (size_t)(buf * kQ9Groups + g) * GE, &qa.tmap, a.gx + tx0 - QS::CO, a.gy + ty0 - P, 3 * g, &BAR[buf]);
+  };
+  if (tid == 0) {
+    issue(blockIdx.x, 0);
+    issue(blockIdx.x + gridDim.x, 1);
+  }
+  // y task: plane yi = 3a + b, column pair yc
+  const bool yon = tid < kN * QT::CP;
+  const int yi = yon ? tid / QT::CP : 0, yc = yon ? tid - yi * QT::CP : 0, yb = yi % kN1;
+  float wy[P][P];
+#pragma unroll
+  for (int l = 0; l < P; ++l)
+#pragma unroll
+    for (int q = 0; q < P; ++q) wy[l][q] = qa.wy[yb][l][q];
+  const bool ybefore = qa.by[yb] != 0;
+  const int ysrc = (yi / 3) * GE + ((yi % 3) * R) * C + C0 + 2 * yc, ydst = yi * (TY / 2) * TW + 2 * yc;
+  // x pass: tail sums of the moving components at this thread's column and its stencil columns
+  int kx = -1;
+  float wx[2][P];
+  const int my_tiles = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+#pragma unroll 1
+  for (int k = 0; k < my_tiles; ++k) {
+    const int tile = blockIdx.x + k * gridDim.x, buf = k & 1;
+    if (k + 1 >= my_tiles) pdl_trigger();
+    const bool late = !mbar_wait(&BAR[buf], (unsigned)((k >> 1) & 1), a.flag);
+    float2* Tb = T + buf * TB;
+    if (yon && !late) {
+      const Store* col = S + (size_t)buf * kQ9Groups * GE + ysrc;
+      float2 win[R];
+#pragma unroll
+      for (int j = 0; j < R; ++j) win[j] = q9_lds2(col + j * C);
+      float2 out[TY];
+      if (yb == 0) {   // at rest along y: the vertex's own row
+#pragma unroll
+        for (int rr = 0; rr < TY; ++rr) out[rr] = win[rr + P];
+      } else {
+#pragma unroll
+        for (int m = 0; m < TY / P; ++m) {
+          // the cell of rows m P .. m P + P - 1 is window rows (m + 1) P .. (m + 2) P; local node 0
+          // takes that cell or the one before
+          float2 d[P], e[P];
+#pragma unroll
+          for (int q = 0; q < P; ++q) {
+            d[q] = sub2(win[(m + 1) * P + q + 1], win[(m + 1) * P + q]);
+            e[q] = sub2(win[m * P + q + 1], win[m * P + q]);
+          }
+#pragma unroll
+          for (int l = 0; l < P; ++l) {
+            float2 acc = (l == 0 && ybefore) ? win[m * P] : win[(m + 1) * P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) acc = fma2(bcast2(wy[l][q]), (l == 0 && ybefore) ? e[q] : d[q], acc);
+            out[m * P + l] = acc;
+          }
+        }
+      }
+      // pairs of rows, two columns in one 16-byte store
+#pragma unroll
+      for (int rr = 0; rr < TY; rr += 2)
+        *reinterpret_cast<float4*>(Tb + ydst + (rr / 2) * TW) = make_float4(out[rr].x, out[rr + 1].x, out[rr].y, out[rr + 1].y);
+    }
+    if (__syncthreads_or(late)) {   // (or the copies of this tile did not land: stop, after those in flight)
+      if (mbar_wait(&BAR[buf], (unsigned)((k >> 1) & 1), a.flag) && k + 1 < my_tiles)
+        mbar_wait(&BAR[buf ^ 1], (unsigned)(((k + 1) >> 1) & 1), a.flag);
+      return;
+    }
+    if (tid == 0) issue(tile + 2 * gridDim.x, buf);   // every thread is done with this buffer
+    const int x = (tile % tiles_x) * 32 + lane, y = (tile / tiles_x) * TY + 2 * rp;
+    if (P == 3 || k == 0) {   // 32 columns are whole cells at p = 1, 2, 4
+      kx = x % P;
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int q = 0; q < P; ++q) wx[c][q] = qa.wx[c + 1][kx][q];
+    }
+    const float2* trow = Tb + rp * TW + (QS::CO - C0) + lane;
+    float2 fb[kN];
+#pragma unroll
+    for (int ca = 0; ca < kN1; ++ca) {
+      const int start = (ca > 0 && kx == 0 && qa.bx[ca]) ? -P : -kx;
+#pragma unroll
+      for (int cb = 0; cb < kN1; ++cb) {
+        const int i = kN1 * ca + cb;
+        const float2* tr = trow + i * (TY / 2) * TW;
+        if (ca == 0) {   // at rest along x
+          fb[i] = tr[0];
+          continue;
+        }
+        float2 v[P + 1];
+        if constexpr (P == 2 || P == 4) {   // even columns: two taps a load
+#pragma unroll
+          for (int q = 0; q < P; q += 2) {
+            const float4 v2 = *reinterpret_cast<const float4*>(tr + start + q);
+            v[q] = make_float2(v2.x, v2.y);
+            v[q + 1] = make_float2(v2.z, v2.w);
+          }
+          v[P] = tr[start + P];
+        } else {
+#pragma unroll
+          for (int q = 0; q <= P; ++q) v[q] = tr[start + q];
+        }
+        float2 acc = v[0];
+#pragma unroll
+        for (int q = 0; q < P; ++q) acc = fma2(bcast2(wx[ca - 1][q]), sub2(v[q + 1], v[q]), acc);
+        fb[i] = acc;
+      }
+    }
+    const bool second = y + 1 < a.ny;
+    if (!second) {   // past the last row: a copy of the first vertex
+#pragma unroll
+      for (int i = 0; i < kN; ++i) fb[i].y = fb[i].x;
+    }
+    const bool ok = collide_q9_pair(fb, a.cs, a.cp);
+    if (x < a.nx && y < a.ny) {
+      if (!ok) atomicOr(a.flag, 1);
+      Store* dst = static_cast<Store*>(a.dst);
+      store_images(a.ghost, x, y, [&](int xx, int yy) {
+        Store* o = dst + (ptrdiff_t)yy * a.pitch + xx;
+#pragma unroll
+        for (int i = 0; i < kN; ++i) st_store(o + (size_t)i * a.plane_stride, fb[i].x);
+      });
+      if (second)
+        store_images(a.ghost, x, y + 1, [&](int xx, int yy) {
+          Store* o = dst + (ptrdiff_t)yy * a.pitch + xx;
+#pragma unroll
+          for (int i = 0; i < kN; ++i) st_store(o + (size_t)i * a.plane_stride, fb[i].y);
+        });
+    }
+  }
+}
+
+template <int P, typename Store>
+static cudaError_t launch_q9_cells(const StepArgs& a, const UniformTables& t, cudaStream_t s) {
+  using QT = Q9Tile<P>;
+  EncodeTiledFn enc = encode_fn();
+  if (!enc) return cudaErrorNotSupported;
+  Q9CellArgs<P> qa;
+  memset(&qa, 0, sizeof(qa));
+  qa.a = a;
+  for (int c = 0; c < kN1; ++c) {
+    for (int l = 0; l < P; ++l)
+      for (int j = 1; j <= P; ++j) {
+        double tx = 0.0, ty = 0.0;
+        for (int m = j; m <= P; ++m) {
+          tx += t.wx_pat[c][l][m];
+          ty += t.wy_pat[c][l][m];
+        }
+        qa.wx[c][l][j - 1] = (float)tx;
+        qa.wy[c][l][j - 1] = (float)ty;
+      }
+    qa.bx[c] = t.dx_pat[c][0] == -P;
+    qa.by[c] = t.dy_pat[c][0] == -P;
+  }
+  const Store* alloc = static_cast<const Store*>(a.src) - ((ptrdiff_t)a.gy * a.pitch + a.gx);
+  const cuuint64_t dims[3] = {(cuuint64_t)a.pitch, (cuuint64_t)a.rows_alloc, (cuuint64_t)kN};
+  const cuuint64_t strides[2] = {(cuuint64_t)a.pitch * sizeof(Store), (cuuint64_t)a.plane_stride * sizeof(Store)};
+  const cuuint32_t box[3] = {(cuuint32_t)Q9Stage<Store>::C, (cuuint32_t)QT::R, 3u};
+  const cuuint32_t estr[3] = {1u, 1u, 1u};
+  const CUtensorMapDataType dt =
+      sizeof(Store) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  if (enc(&qa.tmap, dt, 3, const_cast<Store*>(alloc), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
+      CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  auto kern = step_q9_cell_kernel<P, Store>;
+  constexpr size_t smem = q9_cell_smem<P, Store>();
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int dev = 0, n_sm = 0, per_sm = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, QT::NT, smem)) != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const int ntiles = ((a.nx + 31) / 32) * ((a.ny + QT::TY - 1) / QT::TY);
+  const int grid = ntiles < n_sm * per_sm ? ntiles : n_sm * per_sm;   // persistent CTAs
+  return launch_dependent(kern, dim3(grid), dim3(QT::NT), smem, s, true, qa);
+}
+
+template <int P, typename Store>
+cudaError_t launch_ps(const StepArgs& a, const UniformTables& t, cudaStream_t s) {
+  if constexpr (!std::is_same<Store, double>::value) {
+    if (t.valid) return launch_q9_cells<P, Store>(a, t, s);
+  }
   if constexpr (!std::is_same<Store, double>::value) {
     if (a.q9_tma) {   // chosen (and the ghost images kept) by the host set-up
       Window win;
@@ -673,12 +996,12 @@ cudaError_t launch_ps(const StepArgs& a, cudaStream_t s) {
 }
 
 template <typename Store>
-cudaError_t launch_store(const StepArgs& a, cudaStream_t s) {
+cudaError_t launch_store(const StepArgs& a, const UniformTables& t, cudaStream_t s) {
   switch (a.P) {
-    case 1: return launch_ps<1, Store>(a, s);
-    case 2: return launch_ps<2, Store>(a, s);
-    case 3: return launch_ps<3, Store>(a, s);
-    case 4: return launch_ps<4, Store>(a, s);
+    case 1: return launch_ps<1, Store>(a, t, s);
+    case 2: return launch_ps<2, Store>(a, t, s);
+    case 3: return launch_ps<3, Store>(a, t, s);
+    case 4: return launch_ps<4, Store>(a, t, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -691,12 +1014,12 @@ bool q9_tma_usable(const StepArgs& a, int elem) {
   return q9_tma_window(a, elem, &win, &qt);
 }
 
-cudaError_t launch_step_q9(const StepArgs& a, int store, cudaStream_t s) {
+cudaError_t launch_step_q9(const StepArgs& a, const UniformTables& t, int store, cudaStream_t s) {
   if (a.cs.nq1 != kN1 || a.cp.npop != 1 || a.xs != 1 || a.nv == 0) return cudaErrorInvalidValue;
   switch (store) {
-    case kStoreF32: return launch_store<float>(a, s);
-    case kStoreBF16: return launch_store<__nv_bfloat16>(a, s);
-    case kStoreF64: return launch_store<double>(a, s);
+    case kStoreF32: return launch_store<float>(a, t, s);
+    case kStoreBF16: return launch_store<__nv_bfloat16>(a, t, s);
+    case kStoreF64: return launch_store<double>(a, t, s);
   }
   return cudaErrorInvalidValue;
 }
