@@ -9,7 +9,62 @@ constexpr int kMomThreads = 256;
 
 int moments_blocks(long long nv) { return (int)((nv + kMomThreads - 1) / kMomThreads); }
 
+// Error-free sum: s + x = s' + e exactly, e added to the running error (its own rounding is 2^-24
+// of it: the sum is kept to about 2^-48).
+__device__ __forceinline__ void two_sum(float& s, float& err, float x) {
+  const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+  err = __fadd_rn(err, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
+  s = t;
+}
+
+// rho - 1, j and 2 rho E - 2 C_v of one vertex from its D2Q25 FP32 or BF16 deviations, in FP64: the
+// sums over the velocities of a row, a column and of g in error-free FP32 pairs, combined in FP64
+// (nodes 0, +s, +l, -s, -l).  About 50 FP64 operations a vertex in place of 225, since the FP64 pipe
+// bounds the kernel (1024 x 1024 vertices: 501 -> 168 us, 35 us of traffic), and all 50 loads in
+// flight (32 x 32 vertices: 24.7 -> 18.4 us).
 template <int Store>
+__device__ __forceinline__ void moments25(const MomentArgs& a, size_t o, double* drho, double* jx, double* jy, double* e2) {
+  float rh[kQ1], rl[kQ1], ch[kQ1], cl[kQ1], gh = 0.f, gl = 0.f;
+  const bool two = a.cp.npop == 2;
+#pragma unroll
+  for (int k = 0; k < kQ1; ++k) rh[k] = rl[k] = ch[k] = cl[k] = 0.f;
+#pragma unroll
+  for (int ia = 0; ia < kQ1; ++ia)
+#pragma unroll
+    for (int ib = 0; ib < kQ1; ++ib) {
+      const size_t e = (size_t)(kQ1 * ia + ib) * a.plane_stride + o;
+      float f, g = 0.f;
+      if (Store == kStoreF32) {
+        const float* s = static_cast<const float*>(a.src);
+        f = s[e];
+        if (two) g = s[e + a.ps];
+      } else {
+        const __nv_bfloat16* s = static_cast<const __nv_bfloat16*>(a.src);
+        f = __bfloat162float(s[e]);
+        if (two) g = __bfloat162float(s[e + a.ps]);
+      }
+      two_sum(rh[ia], rl[ia], f);
+      two_sum(ch[ib], cl[ib], f);
+      two_sum(gh, gl, g);
+    }
+  // (an infinite sum has no error term)
+  auto finite = [](float e) { return e == e ? e : 0.f; };
+  double R[kQ1], C[kQ1];
+#pragma unroll
+  for (int k = 0; k < kQ1; ++k) {
+    rl[k] = finite(rl[k]);
+    cl[k] = finite(cl[k]);
+    R[k] = exact_double(rh[k]) + exact_double(rl[k]);
+    C[k] = exact_double(ch[k]) + exact_double(cl[k]);
+  }
+  const double s = a.cs.xi[1], l = a.cs.xi[2], r13 = R[1] + R[3], r24 = R[2] + R[4];
+  *drho = R[0] + r13 + r24;
+  *jx = s * (R[1] - R[3]) + l * (R[2] - R[4]);
+  *jy = s * (C[1] - C[3]) + l * (C[2] - C[4]);
+  *e2 = s * s * (r13 + C[1] + C[3]) + l * l * (r24 + C[2] + C[4]) + (exact_double(gh) + exact_double(finite(gl)));
+}
+
+template <int Store, bool Q25>
 __global__ void __launch_bounds__(kMomThreads) moments_kernel(const __grid_constant__ MomentArgs a) {
   __shared__ double sm[2][kMomThreads];
   const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -20,7 +75,8 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(const __grid_const
     const int npop = a.cp.npop;
     double rho = 0.0, jx = 0.0, jy = 0.0, e2 = 0.0;
     const int nq1 = a.cs.nq1;
-    for (int i = 0; i < nq1 * nq1; ++i) {
+    if constexpr (Q25) moments25<Store>(a, o, &rho, &jx, &jy, &e2);
+    for (int i = 0; i < (Q25 ? 0 : nq1 * nq1); ++i) {
       const double cx = a.cs.xi[i / nq1], cy = a.cs.xi[i % nq1];
       double fv, gv = 0.0;
       if (Store == kStoreF64) {
@@ -45,8 +101,8 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(const __grid_const
       rho += 1.0;
       e2 += 2.0 * a.cp.cv;    // sum w |xi|^2 + K sum w = D + K = 2 C_v
     }
-    const double ux = jx / rho, uy = jy / rho;
-    const double theta = (e2 - rho * (ux * ux + uy * uy)) / (2.0 * a.cp.cv * rho);
+    const double inv = 1.0 / rho, ux = jx * inv, uy = jy * inv;
+    const double theta = (e2 - rho * (ux * ux + uy * uy)) * inv * a.inv2cv;
     if (a.rho) a.rho[v] = (float)rho;
     if (a.u) a.u[v] = (float)ux;
     if (a.v) a.v[v] = (float)uy;
@@ -98,12 +154,21 @@ __global__ void __launch_bounds__(kMomThreads) reduce_partials_kernel(const doub
   }
 }
 
-cudaError_t launch_moments(const MomentArgs& a, cudaStream_t s) {
-  const int blocks = moments_blocks(a.nv);
+cudaError_t launch_moments(const MomentArgs& a0, cudaStream_t s) {
+  const int blocks = moments_blocks(a0.nv);
+  const bool q25 = a0.cs.nq1 == kQ1;
+  MomentArgs a = a0;
+  a.inv2cv = 0.5 / a.cp.cv;
   switch (a.store) {
-    case kStoreF32: moments_kernel<kStoreF32><<<blocks, kMomThreads, 0, s>>>(a); break;
-    case kStoreBF16: moments_kernel<kStoreBF16><<<blocks, kMomThreads, 0, s>>>(a); break;
-    case kStoreF64: moments_kernel<kStoreF64><<<blocks, kMomThreads, 0, s>>>(a); break;
+    case kStoreF32:
+      if (q25) moments_kernel<kStoreF32, true><<<blocks, kMomThreads, 0, s>>>(a);
+      else moments_kernel<kStoreF32, false><<<blocks, kMomThreads, 0, s>>>(a);
+      break;
+    case kStoreBF16:
+      if (q25) moments_kernel<kStoreBF16, true><<<blocks, kMomThreads, 0, s>>>(a);
+      else moments_kernel<kStoreBF16, false><<<blocks, kMomThreads, 0, s>>>(a);
+      break;
+    case kStoreF64: moments_kernel<kStoreF64, false><<<blocks, kMomThreads, 0, s>>>(a); break;
     default: return cudaErrorInvalidValue;
   }
   cudaError_t e = cudaGetLastError();

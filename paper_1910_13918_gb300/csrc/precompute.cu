@@ -253,9 +253,81 @@ __global__ void init_eq_kernel(const __grid_constant__ InitArgs a) {
     }
 }
 
+// The D2Q25 form: mirrored velocity pairs share their even and odd parts (the nodes are 0, +s, +l, -s,
+// -l and He_k(-xi) = (-1)^k He_k(xi)), with the weights folded into the axis factors: about 200 FP64
+// operations a vertex in place of 475, and conversions off the FP64 pipe, which bounds the kernel
+// (1024 x 1024 vertices: 964 -> 412 us; 58 us of traffic).
+template <int Store>
+__global__ void __launch_bounds__(128) init_eq25_kernel(const __grid_constant__ InitArgs a) {
+  const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= a.nv) return;
+  const int iy = (int)(v / a.nx), ix = (int)(v - (long long)iy * a.nx);
+  const double rho = a.rho[v], ux = a.u[v], uy = a.v[v], q = a.T[v] - 1.0;
+  const double x2 = ux * ux, y2 = uy * uy, q3 = 3.0 * q, q6 = 6.0 * q, qq = q3 * q;
+  const double ax[5] = {1.0, ux, x2 + q, ux * (x2 + q3), x2 * (x2 + q6) + qq};
+  const double ay[5] = {1.0, uy, y2 + q, uy * (y2 + q3), y2 * (y2 + q6) + qq};
+  double Xw[5][3];   // rho w_a A_k(u_x) he[k][a]
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    const double r = rho * ax[k];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) Xw[k][c] = (c == 0 && k % 2) ? 0.0 : r * a.wh[k][c];
+  }
+  const double K = a.cp.K, Kq1 = K * (1.0 + q), Kq = K * q, drho = rho - 1.0;
+  const size_t o = (size_t)iy * a.pitch + (size_t)ix * a.xs;
+  auto put = [&](int ia, int ib, double ef, double t) {   // f^eq - w, K q w
+    const int i = kQ1 * ia + ib;
+    const double eg = Kq1 * ef + t;                         // g^eq - K w
+    const size_t of = (size_t)i * a.plane_stride + o;
+    if (Store == kStoreF64) {
+      const double w = a.cs.w[ia] * a.cs.w[ib];
+      double* d = static_cast<double*>(a.dst);
+      d[of] = w + ef;
+      if (a.cp.npop == 2) d[of + a.ps] = K * w + eg;
+    } else if (Store == kStoreF32) {
+      st_pair(static_cast<float*>(a.dst) + of, make_float2(nearest_float(ef), a.cp.npop == 2 ? nearest_float(eg) : 0.f));
+    } else {
+      st_pair(static_cast<__nv_bfloat16*>(a.dst) + of,
+              make_float2(nearest_float(ef), a.cp.npop == 2 ? nearest_float(eg) : 0.f));
+    }
+  };
+#pragma unroll
+  for (int b = 0; b < kQ1; ++b) {
+    const double w = a.cs.w[b];
+    double Sw[5];   // w_b sum_{l <= m} A_l(u_y) he[l][b]
+    Sw[0] = w;
+#pragma unroll
+    for (int m = 1; m <= 4; ++m) {
+      const double h = b < 3 ? a.wh[m][b] : (m % 2 ? -a.wh[m][b - 2] : a.wh[m][b - 2]);
+      Sw[m] = (b == 0 && m % 2) ? Sw[m - 1] : Sw[m - 1] + ay[m] * h;
+    }
+    const double B = w * drho + rho * (Sw[4] - w), t = Kq * w;
+    put(0, b, a.cs.w[0] * B + Xw[2][0] * Sw[2] + Xw[4][0] * Sw[0], a.cs.w[0] * t);
+#pragma unroll
+    for (int c = 1; c <= 2; ++c) {
+      const double ev = a.cs.w[c] * B + Xw[2][c] * Sw[2] + Xw[4][c] * Sw[0];
+      const double od = Xw[1][c] * Sw[3] + Xw[3][c] * Sw[1], tc = a.cs.w[c] * t;
+      put(c, b, ev + od, tc);
+      put(c + 2, b, ev - od, tc);
+    }
+  }
+}
+
 cudaError_t launch_init_equilibrium(const InitArgs& a, cudaStream_t s) {
   const int threads = 128;
   const unsigned blocks = (unsigned)((a.nv + threads - 1) / threads);
+  if (a.cs.nq1 == kQ1) {
+    InitArgs b = a;
+    for (int k = 0; k < kQ1; ++k)
+      for (int c = 0; c < 3; ++c) b.wh[k][c] = a.cs.w[c] * a.cs.he[k][c];
+    switch (a.store) {
+      case kStoreF32: init_eq25_kernel<kStoreF32><<<blocks, threads, 0, s>>>(b); break;
+      case kStoreBF16: init_eq25_kernel<kStoreBF16><<<blocks, threads, 0, s>>>(b); break;
+      case kStoreF64: init_eq25_kernel<kStoreF64><<<blocks, threads, 0, s>>>(b); break;
+      default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+  }
   switch (a.store) {
     case kStoreF32: init_eq_kernel<kStoreF32><<<blocks, threads, 0, s>>>(a); break;
     case kStoreBF16: init_eq_kernel<kStoreBF16><<<blocks, threads, 0, s>>>(a); break;
@@ -324,44 +396,80 @@ cudaError_t launch_ghost_fill(void* origin, int elem, size_t plane_stride, int p
 // ------------------------------------------------------------------------------------------
 // Dense [npop][nq][ny][nx] <-> internal layout (ghost cells, row pitch, interleaved pairs).
 // ------------------------------------------------------------------------------------------
+// A block of 64 x 4 threads takes chunks of 256 columns of 4 rows, a thread 4 columns 64 apart: four
+// coalesced accesses a thread in flight (one a thread held the copies at 4.4 TB/s on 3073 x 3073 vertices,
+// and the index divisions of a flat layout at 1.6 TB/s on the D2Q9 state of 2048 x 2048).
+constexpr int kConvX = 64, kConvY = 4, kConvPer = 4;
+
+static dim3 convert_grid(int nx, int ny, int planes) {
+  const int rows = (ny + kConvY - 1) / kConvY;
+  return dim3((unsigned)((nx + kConvX * kConvPer - 1) / (kConvX * kConvPer)), (unsigned)(rows < 65535 ? rows : 65535),
+              (unsigned)planes);
+}
+
 template <typename E>
-__global__ void state_convert_kernel(const E* src, E* dst, int to_internal, int plane0, int nplanes,
-                                     int nq, int nx, int ny, int pitch, size_t plane_stride, int xs,
-                                     ptrdiff_t ps) {
-  const long long nv = (long long)nx * ny;
-  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t0 >= (long long)nplanes * nv) return;
-  const long long t = t0 + (long long)plane0 * nv;   // index in the dense layout
-  const long long pl = t / nv, v = t - pl * nv;
-  const int pop = (int)(pl / nq), i = (int)(pl - (long long)pop * nq);
-  const int x = (int)(v % nx), y = (int)(v / nx);
-  const ptrdiff_t o = (ptrdiff_t)i * plane_stride + pop * ps + (ptrdiff_t)y * pitch + (ptrdiff_t)x * xs;
-  if (to_internal)
-    dst[o] = src[t];
-  else
-    dst[t] = src[o];
+__global__ void __launch_bounds__(kConvX* kConvY)
+    state_convert_kernel(const E* src, E* dst, int to_internal, int plane0, int nq, int nx, int ny, int pitch,
+                         size_t plane_stride, int xs, ptrdiff_t ps) {
+  const int x0 = blockIdx.x * (kConvX * kConvPer) + threadIdx.x, pl = plane0 + blockIdx.z;
+  const int pop = pl / nq, i = pl - pop * nq;
+  for (int y = blockIdx.y * kConvY + threadIdx.y; y < ny; y += gridDim.y * kConvY) {
+    const size_t d = ((size_t)pl * ny + y) * nx;                                                 // dense row
+    const ptrdiff_t o = (ptrdiff_t)(i * plane_stride) + pop * ps + (ptrdiff_t)y * pitch;      // internal row
+    E v[kConvPer];
+#pragma unroll
+    for (int k = 0; k < kConvPer; ++k) {
+      const int x = x0 + k * kConvX;
+      if (x < nx) v[k] = to_internal ? src[d + x] : src[o + (ptrdiff_t)x * xs];
+    }
+#pragma unroll
+    for (int k = 0; k < kConvPer; ++k) {
+      const int x = x0 + k * kConvX;
+      if (x < nx) {
+        if (to_internal)
+          dst[o + (ptrdiff_t)x * xs] = v[k];
+        else
+          dst[d + x] = v[k];
+      }
+    }
+  }
 }
 
 // Dense [npop][nq][ny][nx] <-> interleaved (f, g) pairs (xs = 2, ps = 1) for the velocity planes
-// i0 .. i0 + gridDim.z - 1: one thread per (plane, vertex), f and g together, so that a pair moves
-// as one 8-byte (FP32) or 4-byte (BF16) access (g = 0 with one population).
+// i0 .. i0 + gridDim.z - 1: f and g together, so that a pair moves as one 8-byte (FP32) or 4-byte
+// (BF16) access (g = 0 with one population).
 template <typename E, typename E2>
-__global__ void pair_convert_kernel(const E* src, E* dst, int to_internal, int i0, int npop, int nq, int nx,
-                                    int ny, int pitch, size_t plane_stride) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, i = i0 + blockIdx.z;
-  if (x >= nx) return;
-  const size_t nv = (size_t)nx * ny;
-  const size_t d = ((size_t)i * ny + y) * nx + x;                            // f in the dense layout
-  const size_t o = (size_t)i * plane_stride + (size_t)y * pitch + 2 * (size_t)x;   // the pair
-  if (to_internal) {
-    E2 p;
-    p.x = src[d];
-    p.y = npop == 2 ? src[(size_t)nq * nv + d] : E(0);
-    *reinterpret_cast<E2*>(dst + o) = p;
-  } else {
-    const E2 p = *reinterpret_cast<const E2*>(src + o);
-    dst[d] = p.x;
-    if (npop == 2) dst[(size_t)nq * nv + d] = p.y;
+__global__ void __launch_bounds__(kConvX* kConvY)
+    pair_convert_kernel(const E* src, E* dst, int to_internal, int i0, int npop, int nq, int nx, int ny, int pitch,
+                        size_t plane_stride) {
+  const int x0 = blockIdx.x * (kConvX * kConvPer) + threadIdx.x, i = i0 + blockIdx.z;
+  const size_t gd = (size_t)nq * nx * ny;   // from f to g in the dense layout
+  for (int y = blockIdx.y * kConvY + threadIdx.y; y < ny; y += gridDim.y * kConvY) {
+    const size_t d = ((size_t)i * ny + y) * nx;                         // f row in the dense layout
+    const size_t o = (size_t)i * plane_stride + (size_t)y * pitch;   // row of pairs
+    E2 p[kConvPer];
+#pragma unroll
+    for (int k = 0; k < kConvPer; ++k) {
+      const int x = x0 + k * kConvX;
+      if (x >= nx) continue;
+      if (to_internal) {
+        p[k].x = src[d + x];
+        p[k].y = npop == 2 ? src[gd + d + x] : E(0);
+      } else {
+        p[k] = *reinterpret_cast<const E2*>(src + o + 2 * (size_t)x);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kConvPer; ++k) {
+      const int x = x0 + k * kConvX;
+      if (x >= nx) continue;
+      if (to_internal) {
+        *reinterpret_cast<E2*>(dst + o + 2 * (size_t)x) = p[k];
+      } else {
+        dst[d + x] = p[k].x;
+        if (npop == 2) dst[gd + d + x] = p[k].y;
+      }
+    }
   }
 }
 
@@ -369,13 +477,13 @@ cudaError_t launch_pair_convert(const void* src, void* dst, bool to_internal, in
                                 int nq, int nx, int ny, int pitch, size_t plane_stride, cudaStream_t s) {
   if (ni == 0) return cudaSuccess;
   if (ny > 65535 || ni > 65535) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)((nx + 255) / 256), (unsigned)ny, (unsigned)ni);
+  const dim3 grid = convert_grid(nx, ny, ni), block(kConvX, kConvY);
   const int ti = to_internal ? 1 : 0;
   if (elem == 4)
-    pair_convert_kernel<uint32_t, uint2><<<grid, 256, 0, s>>>(static_cast<const uint32_t*>(src),
+    pair_convert_kernel<uint32_t, uint2><<<grid, block, 0, s>>>(static_cast<const uint32_t*>(src),
         static_cast<uint32_t*>(dst), ti, i0, npop, nq, nx, ny, pitch, plane_stride);
   else if (elem == 2)
-    pair_convert_kernel<uint16_t, ushort2><<<grid, 256, 0, s>>>(static_cast<const uint16_t*>(src),
+    pair_convert_kernel<uint16_t, ushort2><<<grid, block, 0, s>>>(static_cast<const uint16_t*>(src),
         static_cast<uint16_t*>(dst), ti, i0, npop, nq, nx, ny, pitch, plane_stride);
   else
     return cudaErrorInvalidValue;
@@ -385,23 +493,22 @@ cudaError_t launch_pair_convert(const void* src, void* dst, bool to_internal, in
 cudaError_t launch_state_convert(const void* src, void* dst, bool to_internal, int elem, int plane0,
                                  int nplanes, int nq, int nx, int ny, int pitch, size_t plane_stride,
                                  int xs, ptrdiff_t ps, cudaStream_t s) {
-  const long long n = (long long)nplanes * nx * ny;
-  if (n == 0) return cudaSuccess;
-  const int threads = 256;
-  const unsigned blocks = (unsigned)((n + threads - 1) / threads);
+  if (nplanes == 0) return cudaSuccess;
+  if (nplanes > 65535) return cudaErrorInvalidValue;
+  const dim3 blocks = convert_grid(nx, ny, nplanes), threads(kConvX, kConvY);
   const int ti = to_internal ? 1 : 0;
   switch (elem) {
     case 2:
       state_convert_kernel<uint16_t><<<blocks, threads, 0, s>>>(static_cast<const uint16_t*>(src),
-          static_cast<uint16_t*>(dst), ti, plane0, nplanes, nq, nx, ny, pitch, plane_stride, xs, ps);
+          static_cast<uint16_t*>(dst), ti, plane0, nq, nx, ny, pitch, plane_stride, xs, ps);
       break;
     case 4:
       state_convert_kernel<uint32_t><<<blocks, threads, 0, s>>>(static_cast<const uint32_t*>(src),
-          static_cast<uint32_t*>(dst), ti, plane0, nplanes, nq, nx, ny, pitch, plane_stride, xs, ps);
+          static_cast<uint32_t*>(dst), ti, plane0, nq, nx, ny, pitch, plane_stride, xs, ps);
       break;
     case 8:
       state_convert_kernel<uint64_t><<<blocks, threads, 0, s>>>(static_cast<const uint64_t*>(src),
-          static_cast<uint64_t*>(dst), ti, plane0, nplanes, nq, nx, ny, pitch, plane_stride, xs, ps);
+          static_cast<uint64_t*>(dst), ti, plane0, nq, nx, ny, pitch, plane_stride, xs, ps);
       break;
     default: return cudaErrorInvalidValue;
   }
