@@ -345,7 +345,11 @@ __global__ void __launch_bounds__(kAdjNT, 4) adjoint_stream_tma_kernel(const __g
     }
     const float2* Sm = reinterpret_cast<const float2*>(base + st * SH::kStage);
     const float* Wy = reinterpret_cast<const float*>(Sm + RE);
-    // x pass: target columns cp2, cp2 + 1 of region row r read region columns cp2 .. cp2 + 2H + 1
+    // x pass: target columns cp2, cp2 + 1 of region row r read region columns cp2 .. cp2 + 2H + 1.  A
+    // component at rest has the vertex itself as its only source with weight one: along x the y pass
+    // then reads the region's own columns, along y the row is taken as it is (117 -> 107 us on 1024^2).
+    const bool restx = ia == 0, resty = i - kQ1 * ia == 0;
+    if (!restx)
 #pragma unroll
     for (int j = 0; j < SH::RPW; ++j) {
       const int r = 2 * (warp + j * (kAdjNT / 32)) + half;
@@ -365,12 +369,27 @@ __global__ void __launch_bounds__(kAdjNT, 4) adjoint_stream_tma_kernel(const __g
       }
       *reinterpret_cast<float4*>(Tm + r * kATX + cp2) = make_float4(a0.x, a0.y, a1.x, a1.y);
     }
-    __syncthreads();
+    if (!restx) __syncthreads();   // (the same for the whole CTA)
     // y pass: target rows rr0 .. rr0 + YPW - 1 of column lane read Tm rows rr0 .. rr0 + YPW + 2H - 1
     const int rr0 = SH::YPW * warp, u = x0 + lane;
+    const float2* yin = restx ? Sm + H + lane : Tm + lane;
+    const int yp = restx ? RX : kATX;
+    if (resty) {
+#pragma unroll
+      for (int q = 0; q < SH::YPW; ++q) {
+        const int w = y0 + rr0 + q;
+        if (w < a.ny && u < a.nx) {
+          const float2 v = yin[(rr0 + q + H) * yp];
+          const size_t o = (size_t)w * a.nx + u;
+          a.lam_out[(size_t)i * a.nv + o] = v.x;
+          a.lam_out[(size_t)(kQ + i) * a.nv + o] = has_g ? v.y : 0.f;
+        }
+      }
+      continue;
+    }
     float2 win[SH::YPW + 2 * H];
 #pragma unroll
-    for (int m = 0; m < SH::YPW + 2 * H; ++m) win[m] = Tm[(rr0 + m) * kATX + lane];
+    for (int m = 0; m < SH::YPW + 2 * H; ++m) win[m] = yin[(rr0 + m) * yp];
 #pragma unroll
     for (int q = 0; q < SH::YPW; ++q) {
       const int rr = rr0 + q, w = y0 + rr;
@@ -444,16 +463,25 @@ bool adjoint_tma_usable(int nx, int ny, int periodic_x, int periodic_y, int halo
          (!periodic_y || ny >= 2 * kAdjGhost) && encode_fn() != nullptr;
 }
 
-// S^T on a mapped grid: CSR over the target vertex, per velocity.
+// S^T on a mapped grid: CSR over the target vertex, per velocity, a thread per target.  What bounds it
+// is the lanes' separate rows: each load touches 32 of them.  (A warp reading the contiguous run of
+// its 32 targets' entries side by side and summing through shared memory, and slices of 32 targets
+// padded to one count, are slower all the same: 33.8 and 36.7 us against 26.8 on 257 x 128 vertices,
+// p = 2; the rows are short, 9 entries on average, and counts differ threefold among neighbours.)
 __global__ void __launch_bounds__(256) adjoint_stream_mapped_kernel(const __grid_constant__ AdjointArgs a) {
   const int x = blockIdx.x * 256 + threadIdx.x, i = blockIdx.z;
   if (x >= a.nx) return;
   const float2* m = a.mu + (size_t)i * a.nv;
   const long long* ptr = a.tm_ptr + (size_t)i * (a.nv + 1);
   for (int y = blockIdx.y; y < a.ny; y += gridDim.y) {
-    const long long u = (long long)y * a.nx + x;
+    const long long u = (long long)y * a.nx + x, r0 = ptr[u];
+    const int2* e = a.tm_ent + r0;
+    const int n = (int)(ptr[u + 1] - r0);
     float2 acc = make_float2(0.f, 0.f);
-    for (long long e = ptr[u]; e < ptr[u + 1]; ++e) acc = fma2(bcast2(a.tm_w[e]), __ldg(m + a.tm_col[e]), acc);
+    for (int k = 0; k < n; ++k) {
+      const int2 q = __ldg(e + k);
+      acc = fma2(bcast2(__int_as_float(q.y)), __ldg(m + q.x), acc);
+    }
     a.lam_out[(size_t)i * a.nv + u] = acc.x;
     a.lam_out[(size_t)(kQ + i) * a.nv + u] = (a.cp.npop == 2) ? acc.y : 0.f;
   }

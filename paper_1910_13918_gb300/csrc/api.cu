@@ -90,9 +90,8 @@ struct sllbm_ctx {
   int *tx_deg = nullptr, *ty_deg = nullptr;
   float2* atmp = nullptr;                               // between the x and y passes of S^T
   float *tx_w = nullptr, *ty_w = nullptr;
-  long long* tm_ptr = nullptr;
-  int* tm_col = nullptr;
-  float* tm_w = nullptr;
+  long long* tm_ptr = nullptr;                          // mapped: entries by target
+  int2* tm_ent = nullptr;
   std::vector<void*> allocations;
   std::string err;
 };
@@ -1214,7 +1213,6 @@ static sllbm_status build_mapped_transpose(sllbm_ctx* c) {
   CUDA_TRY(c, cudaMemcpyAsync(r.data(), c->dr64, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(s.data(), c->ds64, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  const int per = (P + 1) * (P + 1);
   std::vector<long long> ptr((size_t)kQ * (nv + 1), 0);
   for (int i = 0; i < kQ; ++i) {
     long long* p0 = &ptr[(size_t)i * (nv + 1)];
@@ -1235,28 +1233,30 @@ static sllbm_status build_mapped_transpose(sllbm_ctx* c) {
     for (long long v = 0; v < nv; ++v) p0[v + 1] += p0[v];
     total = p0[nv];
   }
-  (void)per;
-  std::vector<int> col(total);
-  std::vector<float> wt(total);
+  std::vector<int2> ent(total);
   std::vector<long long> fill(ptr.begin(), ptr.end());
   for (int i = 0; i < kQ; ++i)
     for (long long v = 0; v < nv; ++v) {
       const size_t d = (size_t)i * nv + v;
+      double wx[5], wy[5];
+      for (int k = 0; k <= P; ++k) {
+        wx[k] = lagrange_host(c->ax.nodes, P, k, r[d]);
+        wy[k] = lagrange_host(c->ay.nodes, P, k, s[d]);
+      }
       for (int kb = 0; kb <= P; ++kb)
         for (int ka = 0; ka <= P; ++ka) {
           const int sx = wrap_index(cx[d] * P + ka, nx, c->ax.periodic);
           const int sy = wrap_index(cy[d] * P + kb, ny, c->ay.periodic);
-          const long long e = fill[(size_t)i * (nv + 1) + (long long)sy * nx + sx]++;
-          col[e] = (int)v;
-          wt[e] = (float)(lagrange_host(c->ax.nodes, P, ka, r[d]) * lagrange_host(c->ay.nodes, P, kb, s[d]));
+          int2& e = ent[fill[(size_t)i * (nv + 1) + (long long)sy * nx + sx]++];
+          const float w = (float)(wx[ka] * wy[kb]);
+          e.x = (int)v;
+          memcpy(&e.y, &w, sizeof(float));
         }
     }
   TRY(dalloc(c, &c->tm_ptr, ptr.size()));
-  TRY(dalloc(c, &c->tm_col, (size_t)total));
-  TRY(dalloc(c, &c->tm_w, (size_t)total));
+  TRY(dalloc(c, &c->tm_ent, (size_t)total));
   CUDA_TRY(c, cudaMemcpy(c->tm_ptr, ptr.data(), ptr.size() * sizeof(long long), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(c->tm_col, col.data(), (size_t)total * sizeof(int), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(c->tm_w, wt.data(), (size_t)total * sizeof(float), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpy(c->tm_ent, ent.data(), (size_t)total * sizeof(int2), cudaMemcpyHostToDevice));
   return SLLBM_OK;
 }
 
@@ -1331,8 +1331,7 @@ sllbm_status sllbm_adjoint_step(sllbm_ctx* c, const float* lam_in, float* lam_ou
   a.dhalo = c->thalo_k;
   a.dw = c->tdw;
   a.tm_ptr = c->tm_ptr;
-  a.tm_col = c->tm_col;
-  a.tm_w = c->tm_w;
+  a.tm_ent = c->tm_ent;
   CUDA_TRY(c, launch_adjoint_step(a, c->stream));
   return SLLBM_OK;
 }

@@ -222,9 +222,8 @@ struct AdjointArgs {
   const float* tx_dense;
   const float* ty_dense;
   int dhalo, dw;
-  const long long* tm_ptr;  // [25][nv+1]
-  const int* tm_col;
-  const float* tm_w;
+  const long long* tm_ptr;  // [25][nv+1]: first entry of each target
+  const int2* tm_ent;       // (vertex, weight)
 };
 cudaError_t launch_adjoint_step(const AdjointArgs& a, cudaStream_t s);
 // Ghost width of the pairs of the one-pass S^T (its largest transposed-stencil halo), and whether
