@@ -120,16 +120,19 @@ __host__ __device__ __forceinline__ int wrap_index(int j, int n, int periodic) {
 // FP64 on few FP64 instructions: that pipe adds, multiplies and converts two values a clock and SM.
 // The exact double of a float, in integer instructions (the FP64 pipe converts and adds at a
 // sixty-fourth of the FP32 rate); zeros, subnormals and non-finite values convert as usual.
+// (The rare cases are calls, so that the conversion instruction is not issued for every value.)
+static __device__ __noinline__ double convert_double(float x) { return (double)x; }
+static __device__ __noinline__ float convert_float(double x) { return (float)x; }
 __device__ __forceinline__ double exact_double(float x) {
   const unsigned b = __float_as_uint(x), e = b & 0x7fffffffu;
-  if (e - 0x00800000u >= 0x7f000000u) return (double)x;
+  if (e - 0x00800000u >= 0x7f000000u) return convert_double(x);
   return __hiloint2double((int)((b & 0x80000000u) | ((e >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
 // A double rounded to the nearest float (ties to even), likewise in integer instructions.
 __device__ __forceinline__ float nearest_float(double d) {
   const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  if (((hi >> 20) & 0x7ffu) - 897u >= 254u) return (float)d;   // not a normal float
+  if (((hi >> 20) & 0x7ffu) - 897u >= 254u) return convert_float(d);   // not a normal float
   unsigned m = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
   const unsigned rest = lo & 0x1fffffffu;
   m += rest > 0x10000000u || (rest == 0x10000000u && (m & 1u));
