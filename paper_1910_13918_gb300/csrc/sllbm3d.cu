@@ -543,6 +543,11 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
       for (int c = 0; c < ZR; ++c) {
         const int t = tid + c * NT;
         if (t < SH::ZT) {
+          if (zc == 0) {   // at rest along z: the vertex's own slice
+#pragma unroll
+            for (int tz = 0; tz < TZ; ++tz) zout[tz * SH::ZS + t] = Sst[(tz + P) * RY * RX + t];
+            continue;
+          }
           float2 v[RZ], d[RZ - 1];
 #pragma unroll
           for (int r = 0; r < RZ; ++r) v[r] = Sst[r * RY * RX + t];
@@ -564,13 +569,18 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
         const float* wy = Wy + yb * kT3Y * NW;
         const float2* zin = Zb + ((i - 1) & 1) * SH::ZB + ytz * SH::ZS + ycol;
         float2* yout = Yb + ((i - 1) & 1) * SH::YB + ytz * SH::YS + ycol;
-        float2 v[RY], d[RY - 1];
+        if (yb == 0) {   // at rest along y
 #pragma unroll
-        for (int r = 0; r < RY; ++r) v[r] = zin[r * RX];
+          for (int ty = 0; ty < kT3Y; ++ty) yout[ty * RX] = zin[(ty + P) * RX];
+        } else {
+          float2 v[RY], d[RY - 1];
 #pragma unroll
-        for (int r = 0; r + 1 < RY; ++r) d[r] = sub2(v[r + 1], v[r]);
+          for (int r = 0; r < RY; ++r) v[r] = zin[r * RX];
 #pragma unroll
-        for (int ty = 0; ty < kT3Y; ++ty) yout[ty * RX] = tail_interp<P>(v, d, ty + P, wy + ty * NW);
+          for (int r = 0; r + 1 < RY; ++r) d[r] = sub2(v[r + 1], v[r]);
+#pragma unroll
+          for (int ty = 0; ty < kT3Y; ++ty) yout[ty * RX] = tail_interp<P>(v, d, ty + P, wy + ty * NW);
+        }
       }
       if (++yc == kQ1) {
         yc = 0;
@@ -592,16 +602,24 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
         const int row = (tid + k * NT) >> 4;
         const float4* in = reinterpret_cast<const float4*>(Yb + (i & 1) * SH::YB + (row / kT3Y) * SH::YS +
                                                            (row % kT3Y) * RX + 2 * xp);
-        float2 v[2 * XO + 2], d[2 * XO + 1];
+        float2 r0, r1;
+        if (xa == 0) {   // at rest along x
+          const float4 q = in[XO / 2];
+          r0 = make_float2(q.x, q.y);
+          r1 = make_float2(q.z, q.w);
+        } else {
+          float2 v[2 * XO + 2], d[2 * XO + 1];
 #pragma unroll
-        for (int j = 0; j <= XO; ++j) {
-          const float4 q = in[j];
-          v[2 * j] = make_float2(q.x, q.y);
-          v[2 * j + 1] = make_float2(q.z, q.w);
+          for (int j = 0; j <= XO; ++j) {
+            const float4 q = in[j];
+            v[2 * j] = make_float2(q.x, q.y);
+            v[2 * j + 1] = make_float2(q.z, q.w);
+          }
+#pragma unroll
+          for (int j = 0; j < 2 * XO + 1; ++j) d[j] = sub2(v[j + 1], v[j]);
+          r0 = tail_interp<P>(v, d, XO, wx[0]);
+          r1 = tail_interp<P>(v, d, XO + 1, wx[1]);
         }
-#pragma unroll
-        for (int j = 0; j < 2 * XO + 1; ++j) d[j] = sub2(v[j + 1], v[j]);
-        const float2 r0 = tail_interp<P>(v, d, XO, wx[0]), r1 = tail_interp<P>(v, d, XO + 1, wx[1]);
         if (on[k]) {
           if (both)
             *reinterpret_cast<float4*>(out[k]) = make_float4(r0.x, r0.y, r1.x, r1.y);
