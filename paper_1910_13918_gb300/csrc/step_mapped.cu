@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(kMNT, 2) step_mapped_kernel(const __grid_const
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   __syncthreads();
+  pdl_wait();   // the step before has written the source and is done with the destination
 
   // stage st of a tile = planes 5 st .. 5 st + 4, one window copy each; global stage counter as
   // in the uniform kernel
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kMNT, 2) step_mapped_kernel(const __grid_const
   long s0 = 0;
 #pragma unroll 1
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, s0 += kQ1) {
+    if (tile + (int)gridDim.x >= ntiles) pdl_trigger();   // its last tile: what follows may take its place
     const int x = (tile % tiles_x) * kMappedTileX + lane, y = (tile / tiles_x) * kMappedTileY + row;
     const bool store = x < a.nx && y < a.ny && __ldg(ma.tile_ok + tile);
     float2 fg[kQ];
@@ -242,8 +244,8 @@ static cudaError_t launch_p(const StepArgs& a, const MappedTables& t, cudaStream
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int ntiles = ((a.nx + kMappedTileX - 1) / kMappedTileX) * ((a.ny + kMappedTileY - 1) / kMappedTileY);
   const int grid = ntiles < n_sm * per_sm ? ntiles : n_sm * per_sm;   // persistent CTAs
-  step_mapped_kernel<P, Store, PR><<<grid, kMNT, smem, s>>>(ma);
-  return cudaGetLastError();
+  // the set-up of a step overlaps the end of the step before
+  return launch_dependent(step_mapped_kernel<P, Store, PR>, dim3(grid), dim3(kMNT), smem, s, true, ma);
 }
 
 template <typename Store>
