@@ -25,11 +25,13 @@ class SLLBMRollout(torch.autograd.Function):
     def forward(ctx, u0, v0, sim: SLLBM, rho0, T0, nsteps: int, k: int):
         with torch.cuda.stream(sim._stream):
             sim.init(rho0, u0, v0, T0)
-            checkpoints = {0: sim.get_state().clone()}
-            for n in range(nsteps):
-                sim.step(1)
-                if (n + 1) % k == 0 and n + 1 < nsteps:
-                    checkpoints[n + 1] = sim.get_state().clone()
+            # a segment a call: get_state returns a tensor of its own, and small states replay the
+            # step's graph within a call
+            checkpoints = {0: sim.get_state()}
+            for start in range(0, nsteps, k):
+                sim.step(min(k, nsteps - start))
+                if start + k < nsteps:
+                    checkpoints[start + k] = sim.get_state()
             rho = sim.moments(sums=False)["rho"].double()
         ctx.sim, ctx.nsteps, ctx.k, ctx.checkpoints = sim, nsteps, k, checkpoints
         ctx.save_for_backward(u0, v0, rho0, T0)

@@ -513,7 +513,7 @@ cudaError_t launch_adjoint_step(const AdjointArgs& a, cudaStream_t s) {
 // d/du of <lambda, (f^eq, g^eq)(rho, u, v, theta)> per vertex, in FP64: through the Hermite moments
 // M[k][l] of lambda^f + K theta lambda^g (as adjoint_z), the sums taken over mirrored nodes first
 // (0, +s, +l, -s, -l: even and odd parts): about 220 FP64 operations a vertex, the pipe that bounds it,
-// in place of 25 evaluations of E and its derivatives (1024 x 1024 vertices: 1106 -> 525 us).
+// in place of 25 evaluations of E and its derivatives (1024 x 1024 vertices: 1106 -> 440 us).
 __global__ void __launch_bounds__(128) init_vjp_kernel(const __grid_constant__ InitVjpArgs a) {
   const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= a.nv) return;

@@ -20,8 +20,8 @@ __device__ __forceinline__ void two_sum(float& s, float& err, float x) {
 // rho - 1, j and 2 rho E - 2 C_v of one vertex from its D2Q25 FP32 or BF16 deviations, in FP64: the
 // sums over the velocities of a row, a column and of g in error-free FP32 pairs, combined in FP64
 // (nodes 0, +s, +l, -s, -l).  About 50 FP64 operations a vertex in place of 225, since the FP64 pipe
-// bounds the kernel (1024 x 1024 vertices: 501 -> 168 us, 35 us of traffic), and all 50 loads in
-// flight (32 x 32 vertices: 24.7 -> 18.4 us).
+// bounds the kernel (1024 x 1024 vertices: 501 -> 119 us, 35 us of traffic), and all 50 loads in
+// flight (32 x 32 vertices: 24.7 -> 14.3 us).
 template <int Store>
 __device__ __forceinline__ void moments25(const MomentArgs& a, size_t o, double* drho, double* jx, double* jy, double* e2) {
   float rh[kQ1], rl[kQ1], ch[kQ1], cl[kQ1], gh = 0.f, gl = 0.f;

@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__
 // images of the vertices next to periodic faces.
 //
 // What bounds it: the latency of the phases and shared memory together (64^3: the LSU pipe at 65 %,
-// issue at 39 %; 128^3: 1.205 ms, 1.38 ms with three barriers a plane and one vertex a task).  Deeper
+// issue at 39 %; 128^3: 1.187 ms, 1.38 ms with three barriers a plane and one vertex a task).  Deeper
 // tiles (32 x 8 x 8, three stages, one CTA of 512 threads) take the same time; 24 warps an SM on
 // tiles of 3 or 2 slices take 1.50 and 1.44 ms, as their regions grow.  250 values a vertex rule out a
 // collision in registers, so the two kernels move 16 bytes an update.
@@ -915,7 +915,7 @@ __global__ void __launch_bounds__(128) tail_table_kernel(const int* off, const d
 
 // FP32 pairs (layout lay) <-> dense FP64 full populations [npop][125][nv]: plane i = blockIdx.y, whose
 // lattice weights the block forms once.  (With four FP64 products a value and FP64 conversions the
-// FP64 pipe bound it: 2.94 ms for the 2.1 M vertices of 128^3, now 1.37 ms, 0.95 ms of it HBM traffic.)
+// FP64 pipe bound it: 2.94 ms for the 2.1 M vertices of 128^3, now 1.27 ms in and 1.31 out, 0.95 ms of it HBM traffic.)
 constexpr int kConvPer = 4;   // vertices a thread
 __global__ void __launch_bounds__(256) convert3d_kernel(float2* pairs, Pad3 lay, double* dense, int nx, int ny,
                                                         unsigned nv, int npop, double K, const __grid_constant__ Consts cs,
