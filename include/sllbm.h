@@ -240,7 +240,7 @@ sllbm_status sllbm_selftest_bounded_wait(void* cuda_stream);
  * with the same fourth-order equilibrium (Sec. II.A over index tuples in {x, y, z}^n), g^eq =
  * (2 C_v - 3) theta f^eq (Sec. II.D) and BGK (Eq. streaming_fg, Pr = 1).  params.velset =
  * SLLBM_VEL_D3Q125 with params.prec = SLLBM_PREC_F64_PLAIN (plain FP64 step on full populations)
- * or SLLBM_PREC_F32 (fused FP32 step: one launch per step, the state kept as FP32 deviations
+ * or SLLBM_PREC_F32 (FP32 step, see sllbm3d_step; the state kept as FP32 deviations
  * (f - w, g - K w) side by side; get_state / set_state still exchange FP64 full populations);
  * pr 0 or 1, cv >= 3/2 (cv = 3/2 carries f only; isothermal = 1 needs it).  Population field
  * [n_pop][125][nz][ny][nx], velocity i = 25a + 5b + c (D1Q5 indices of the x, y, z components in
@@ -271,12 +271,13 @@ sllbm_status sllbm3d_precompute_departures(sllbm3d_ctx* ctx);
 sllbm_status sllbm3d_init_equilibrium(sllbm3d_ctx* ctx, const double* rho_dev, const double* u_dev,
                                       const double* v_dev, const double* w_dev, const double* T_dev);
 /* Advance nsteps steps (pull interpolation of every velocity with the tensor-product Lagrange
- * basis, moments, BGK); enqueues only.  FP32 contexts of order 1 or 2 with an even number of x
- * vertices and at least 36 x 12 x 8 vertices take the sum-factorised step (three launches:
- * TMA-staged tiles that interpolate and sum the moments, a sweep that relaxes, a refresh of the
- * periodic images in the state's ghost cells); the others the one-launch gather step.  The
- * sum-factorised step keeps 2 ghost cells on every axis in its state and allocates 6 floats a
- * vertex of scratch at sllbm3d_precompute_departures. */
+ * basis, moments, BGK); enqueues only.  FP32 contexts on grids of at least 36 x 12 x 8 vertices whose
+ * departures stay within the neighbouring cells (and, on periodic axes, with three cells or more)
+ * take the sum-factorised step (two launches: TMA-staged tiles that interpolate and sum the moments,
+ * a sweep that relaxes and writes the periodic images in the state's ghost cells); the others the
+ * one-launch gather step.  The sum-factorised step keeps 2 (orders 1, 2) or 4 ghost cells on every
+ * axis in its state and allocates 6 floats a vertex of scratch at sllbm3d_precompute_departures.
+ */
 sllbm_status sllbm3d_step(sllbm3d_ctx* ctx, int nsteps);
 /* Name of the kernel sllbm3d_step uses for this context ("stream3d" for the sum-factorised FP32
  * step, "gather_f32", "plain_f64"); valid after sllbm3d_precompute_departures. */
