@@ -42,12 +42,13 @@ SECONDARY = "tgv256"          # second grid of the line: the Taylor-Green vortex
 # DRAM traffic (read + write bytes per launch) of the step kernel from an ncu capture, keyed by
 # (kernel source digest, workload, precision); reported as null once the kernel source changes.
 NCU_TRAFFIC = {
-    # 512^2-cell capture: 511.6 MB read + 429.2 MB written for 2,362,369 vertices, scaled by the
-    # vertex count to the 3073^2 grid (a multi-pass capture of that grid exceeds the size rule)
-    ("99a5f9bcc84ce154", "riemann1024_p3_tableIII", "f32"): 940.84e6 * 9443329 / 2362369,
-    ("99a5f9bcc84ce154", "riemann512_p3_tableIII", "f32"): 940.84e6,
-    # full-size capture: 219.5 MB read + 174.1 MB written
-    ("99a5f9bcc84ce154", "tgv256_p4", "f32"): 393.62e6,
+    # 512^2-cell capture, both launches of a step (interior tiles 484.1 MB read + 415.9 MB written,
+    # edge tiles 38.2 MB read, their writes still in L2), 2,362,369 vertices, scaled by the vertex count
+    # to the 3073^2 grid (a multi-pass capture of that grid exceeds the size rule)
+    ("063a83de6c004d8b", "riemann1024_p3_tableIII", "f32"): 938.24e6 * 9443329 / 2362369,
+    ("063a83de6c004d8b", "riemann512_p3_tableIII", "f32"): 938.24e6,
+    # full-size capture: 217.7 MB read + 170.3 MB written
+    ("063a83de6c004d8b", "tgv256_p4", "f32"): 388.0e6,
 }
 
 # Sources that decide what the fused kernels of NCU_TRAFFIC do and how they are launched on
