@@ -196,8 +196,13 @@ __device__ __forceinline__ int wrap1(int j, int n, int periodic) {
 // equilibrium and sums the residual moments of (f^eq - f); the residuals (the FP32 rounding of
 // the equilibrium) are then removed at the rest velocity and at (s, 0, 0), (0, s, 0), (0, 0, s)
 // for mass and momentum, and on g at the rest velocity for the energy.
-template <int P>
-__global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__ Step3F32Args a) {
+// Two forms. Grids of one wave (4 blocks an SM): the registers go to the (p+1)^3 gathers in flight, which
+// such a grid waits for, and f^eq - w is summed by order without its leading 1 (18 x 22 x 28 vertices, p = 2:
+// 109 us a step, 130 in the other form; 20 x 36 x 80, p = 4: 458 and 595).  Larger grids (no bound): more warps
+// share L1 and L2, and the nested sum, whose products hide the loads of the second sweep, is the
+// faster one (96^3, p = 4, departures beyond the neighbouring cells: 5.95 ms, 6.33 with the sum by order and 7 blocks).
+template <int P, int BLOCKS>
+__global__ void __launch_bounds__(128, BLOCKS) step3d_f32_kernel(const __grid_constant__ Step3F32Args a) {
   const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= a.nv) return;
   const int ix = (int)(v % a.nx);
@@ -276,13 +281,13 @@ __global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__
       A3[d][4] = u * u * (u * u + 6.f * q) + 3.f * q * q;
     }
   }
-  float Zc[5][5];   // [n][c], compile-time indices only
+  float Zc[5][5];   // [n][c], compile-time indices only (with the leading 1 in the nested form)
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     float acc = 0.f;
-    Zc[0][c] = 0.f;
+    if constexpr (BLOCKS == 4) Zc[0][c] = 0.f;
 #pragma unroll
-    for (int m = 1; m < 5; ++m) {
+    for (int m = BLOCKS == 4 ? 1 : 0; m < 5; ++m) {
       acc += Az[m] * a.cs.hef[m][c];
       Zc[m][c] = acc;
     }
@@ -309,9 +314,22 @@ __global__ void __launch_bounds__(128) step3d_f32_kernel(const __grid_constant__
 #pragma unroll
       for (int ic = 0; ic < kQ1; ++ic) {
         const int i = 25 * ia + 5 * ib + ic;
-        const float em1 = fmaf(C1, Zc[1][ic], fmaf(C2, Zc[2][ic], fmaf(C3, Zc[3][ic], Cs + Zc[4][ic])));
+        float em1;
+        if constexpr (BLOCKS == 4) {
+          em1 = fmaf(C1, Zc[1][ic], fmaf(C2, Zc[2][ic], fmaf(C3, Zc[3][ic], Cs + Zc[4][ic])));
+        } else {
+          float s1 = 0.f;
+#pragma unroll
+          for (int k = 0; k <= 4; ++k) {
+            float sl = 0.f;
+#pragma unroll
+            for (int l = 0; l <= 4 - k; ++l) sl += Yb[l] * Zc[4 - k - l][ic];
+            s1 += Xa[k] * sl;
+          }
+          em1 = s1 - 1.f;
+        }
         const float w = wab * a.cs.wf[ic];
-        const float ef = w * fmaf(rho, em1, drho);
+        const float ef = BLOCKS == 4 ? w * fmaf(rho, em1, drho) : w * (drho + rho * em1);
         const float eg = Kq1 * ef + Kq * w;   // g^eq - K w = K ((1 + q)(f^eq - w) + q w)
         float2* o = a.dst + (size_t)i * plane + v;
         const float2 fg = *o;
@@ -1443,11 +1461,20 @@ sllbm_status sllbm3d_step(sllbm3d_ctx* c, int nsteps) {
       }
       b.src = pairs(c, c->cur);
       b.dst = pairs(c, c->cur ^ 1);
-      switch (c->g.order) {
-        case 1: step3d_f32_kernel<1><<<blocks, 128, 0, c->stream>>>(b); break;
-        case 2: step3d_f32_kernel<2><<<blocks, 128, 0, c->stream>>>(b); break;
-        case 3: step3d_f32_kernel<3><<<blocks, 128, 0, c->stream>>>(b); break;
-        default: step3d_f32_kernel<4><<<blocks, 128, 0, c->stream>>>(b); break;
+      if (blocks <= 4 * 152) {   // one wave
+        switch (c->g.order) {
+          case 1: step3d_f32_kernel<1, 4><<<blocks, 128, 0, c->stream>>>(b); break;
+          case 2: step3d_f32_kernel<2, 4><<<blocks, 128, 0, c->stream>>>(b); break;
+          case 3: step3d_f32_kernel<3, 4><<<blocks, 128, 0, c->stream>>>(b); break;
+          default: step3d_f32_kernel<4, 4><<<blocks, 128, 0, c->stream>>>(b); break;
+        }
+      } else {
+        switch (c->g.order) {
+          case 1: step3d_f32_kernel<1, 0><<<blocks, 128, 0, c->stream>>>(b); break;
+          case 2: step3d_f32_kernel<2, 0><<<blocks, 128, 0, c->stream>>>(b); break;
+          case 3: step3d_f32_kernel<3, 0><<<blocks, 128, 0, c->stream>>>(b); break;
+          default: step3d_f32_kernel<4, 0><<<blocks, 128, 0, c->stream>>>(b); break;
+        }
       }
       const sllbm_status s = cuda3(c, cudaGetLastError(), "step3d_f32_kernel");
       if (s != SLLBM_OK) return s;
