@@ -197,10 +197,12 @@ __device__ __forceinline__ int wrap1(int j, int n, int periodic) {
 // the equilibrium) are then removed at the rest velocity and at (s, 0, 0), (0, s, 0), (0, 0, s)
 // for mass and momentum, and on g at the rest velocity for the energy.
 // Two forms. Grids of one wave (4 blocks an SM): the registers go to the (p+1)^3 gathers in flight, which
-// such a grid waits for, and f^eq - w is summed by order without its leading 1 (18 x 22 x 28 vertices, p = 2:
+// such a grid waits for, and f^eq - w is summed by order (18 x 22 x 28 vertices, p = 2:
 // 109 us a step, 130 in the other form; 20 x 36 x 80, p = 4: 458 and 595).  Larger grids (no bound): more warps
 // share L1 and L2, and the nested sum, whose products hide the loads of the second sweep, is the
-// faster one (96^3, p = 4, departures beyond the neighbouring cells: 5.95 ms, 6.33 with the sum by order and 7 blocks).
+// faster one (96^3, p = 4, departures beyond the neighbouring cells: 6.10 ms, 6.33 with the sum by order and 7 blocks).
+// Neither forms the leading 1 of the sum and takes it off afterwards: that left its rounding on every
+// value (44^3, deviations of 1e-4 of the weights: 6e-3 of the largest deviation in one step, 3e-6 now).
 template <int P, int BLOCKS>
 __global__ void __launch_bounds__(128, BLOCKS) step3d_f32_kernel(const __grid_constant__ Step3F32Args a) {
   const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -281,16 +283,19 @@ __global__ void __launch_bounds__(128, BLOCKS) step3d_f32_kernel(const __grid_co
       A3[d][4] = u * u * (u * u + 6.f * q) + 3.f * q * q;
     }
   }
-  float Zc[5][5];   // [n][c], compile-time indices only (with the leading 1 in the nested form)
+  // (nested: sum_k X_k sum_l Y_l (1 + Zc_{4-k-l}), the term k = l = 0 being Zc_4 alone)
+  float Zc[5][5], Z4[5];   // [n][c] and Zc_4, compile-time indices only (nested: 1 + Zc_n)
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
-    float acc = 0.f;
+    float acc = 0.f, z = 0.f;
     if constexpr (BLOCKS == 4) Zc[0][c] = 0.f;
 #pragma unroll
     for (int m = BLOCKS == 4 ? 1 : 0; m < 5; ++m) {
       acc += Az[m] * a.cs.hef[m][c];
+      if (m > 0) z += Az[m] * a.cs.hef[m][c];
       Zc[m][c] = acc;
     }
+    Z4[c] = z;
   }
   const float om = a.omega, Kq1 = a.K * (1.f + q), Kq = a.K * q;
   const float2 om2 = bcast2(om);
@@ -316,20 +321,19 @@ __global__ void __launch_bounds__(128, BLOCKS) step3d_f32_kernel(const __grid_co
         const int i = 25 * ia + 5 * ib + ic;
         float em1;
         if constexpr (BLOCKS == 4) {
-          em1 = fmaf(C1, Zc[1][ic], fmaf(C2, Zc[2][ic], fmaf(C3, Zc[3][ic], Cs + Zc[4][ic])));
+          em1 = fmaf(C1, Zc[1][ic], fmaf(C2, Zc[2][ic], fmaf(C3, Zc[3][ic], Cs + Z4[ic])));
         } else {
-          float s1 = 0.f;
+          em1 = 0.f;
 #pragma unroll
           for (int k = 0; k <= 4; ++k) {
-            float sl = 0.f;
+            float sl = k == 0 ? Z4[ic] : 0.f;
 #pragma unroll
-            for (int l = 0; l <= 4 - k; ++l) sl += Yb[l] * Zc[4 - k - l][ic];
-            s1 += Xa[k] * sl;
+            for (int l = k == 0 ? 1 : 0; l <= 4 - k; ++l) sl += Yb[l] * Zc[4 - k - l][ic];
+            em1 += Xa[k] * sl;
           }
-          em1 = s1 - 1.f;
         }
         const float w = wab * a.cs.wf[ic];
-        const float ef = BLOCKS == 4 ? w * fmaf(rho, em1, drho) : w * (drho + rho * em1);
+        const float ef = w * fmaf(rho, em1, drho);
         const float eg = Kq1 * ef + Kq * w;   // g^eq - K w = K ((1 + q)(f^eq - w) + q w)
         float2* o = a.dst + (size_t)i * plane + v;
         const float2 fg = *o;
