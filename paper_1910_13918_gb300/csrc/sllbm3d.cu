@@ -1105,6 +1105,7 @@ struct sllbm3d_ctx {
   Consts cs{};
   int npop = 2;
   bool f32 = false;                      // FP32 deviation pairs (else FP64 full populations)
+  int n_sm = 0;                          // of the device
   long long nv = 0;
   double* state[2] = {nullptr, nullptr}; // FP32: reinterpreted as float2 [125][nv]
   int cur = 0;
@@ -1293,6 +1294,11 @@ sllbm_status sllbm3d_create(const sllbm_grid3_desc* g, const sllbm_params* p, vo
   c->nv = (long long)c->ax.nv * c->ay.nv * c->az.nv;
   c->npop = p->cv == 1.5 ? 1 : 2;
   c->f32 = p->prec == SLLBM_PREC_F32;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();   // (no device: the allocations below fail)
+    c->n_sm = 0;
+  }
   c->tiled = tiled3d_usable(c, p->dt);   // its state keeps ghost cells, in rows of whole 16-byte units
   {
     Pad3& L = c->lay;
@@ -1465,7 +1471,7 @@ sllbm_status sllbm3d_step(sllbm3d_ctx* c, int nsteps) {
       }
       b.src = pairs(c, c->cur);
       b.dst = pairs(c, c->cur ^ 1);
-      if (blocks <= 4 * 152) {   // one wave
+      if (blocks <= 4u * (unsigned)c->n_sm) {   // one wave
         switch (c->g.order) {
           case 1: step3d_f32_kernel<1, 4><<<blocks, 128, 0, c->stream>>>(b); break;
           case 2: step3d_f32_kernel<2, 4><<<blocks, 128, 0, c->stream>>>(b); break;
