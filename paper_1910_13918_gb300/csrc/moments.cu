@@ -9,59 +9,78 @@ constexpr int kMomThreads = 256;
 
 int moments_blocks(long long nv) { return (int)((nv + kMomThreads - 1) / kMomThreads); }
 
-// Error-free sum: s + x = s' + e exactly, e added to the running error (its own rounding is 2^-24
-// of it: the sum is kept to about 2^-48).
-__device__ __forceinline__ void two_sum(float& s, float& err, float x) {
-  const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
-  err = __fadd_rn(err, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
-  s = t;
-}
+// A value as three FP32 parts, the first two rounded to the same units for all values of a sum, 2^-18 and
+// 2^-38 of a power of two 2^E at most the largest magnitude: their sums (25 values, in any order and with
+// any signs) are exact, and those of the rest, below 2^-39 2^E a value, round at 2^-59 2^E.  So the whole sum
+// is good to 2^-54 of the largest value, where adding in FP64 rounds each partial sum at 2^-53 of it.
+// (Extraction of leading parts: Rump, Ogita and Oishi, Accurate floating-point summation.)
+struct Parts {
+  float a = 0.f, b = 0.f, c = 0.f;
+  __device__ __forceinline__ double value() const { return exact_double(a) + (exact_double(b) + exact_double(c)); }
+};
+__device__ __forceinline__ Parts operator+(const Parts& x, const Parts& y) { return {x.a + y.a, x.b + y.b, x.c + y.c}; }
+__device__ __forceinline__ Parts operator-(const Parts& x, const Parts& y) { return {x.a - y.a, x.b - y.b, x.c - y.c}; }
+
+struct PartUnits {   // 1.5 2^(E + 5) and 1.5 2^(E - 15): adding them rounds to the units
+  float s1, s2;
+  __device__ __forceinline__ explicit PartUnits(float largest) {
+    const float p = __uint_as_float(__float_as_uint(fmaxf(largest, 0x1p-100f)) & 0x7f800000u);
+    s1 = p * 48.f;
+    s2 = p * (48.f / 0x1p20f);
+  }
+  __device__ __forceinline__ Parts split(float x) const {
+    const float q = __fsub_rn(__fadd_rn(x, s1), s1), r = __fsub_rn(x, q), t = __fsub_rn(__fadd_rn(r, s2), s2);
+    return {q, t, __fsub_rn(r, t)};
+  }
+};
 
 // rho - 1, j and 2 rho E - 2 C_v of one vertex from its D2Q25 FP32 or BF16 deviations, in FP64: the
-// sums over the velocities of a row, a column and of g in error-free FP32 pairs, combined in FP64
-// (nodes 0, +s, +l, -s, -l).  About 50 FP64 operations a vertex in place of 225, since the FP64 pipe
+// sums over the velocities in FP32 parts, combined in FP64 (nodes 0, +s, +l, -s, -l).  About 55 FP64
+// operations a vertex in place of 225, since the FP64 pipe
 // bounds the kernel (1024 x 1024 vertices: 501 -> 119 us, 35 us of traffic), and all 50 loads in
-// flight (32 x 32 vertices: 24.7 -> 14.3 us).
+// flight (32 x 32 vertices: 24.7 -> 14.3 us).  False if a value is not finite or a sum might leave the FP32
+// range: the caller then sums in FP64.
 template <int Store>
-__device__ __forceinline__ void moments25(const MomentArgs& a, size_t o, double* drho, double* jx, double* jy, double* e2) {
-  float rh[kQ1], rl[kQ1], ch[kQ1], cl[kQ1], gh = 0.f, gl = 0.f;
+__device__ __forceinline__ bool moments25(const MomentArgs& a, size_t o, double* drho, double* jx, double* jy, double* e2) {
+  float f[kQ], g[kQ], fm = 0.f, gm = 0.f;
   const bool two = a.cp.npop == 2;
 #pragma unroll
-  for (int k = 0; k < kQ1; ++k) rh[k] = rl[k] = ch[k] = cl[k] = 0.f;
+  for (int i = 0; i < kQ; ++i) {
+    const size_t e = (size_t)i * a.plane_stride + o;
+    g[i] = 0.f;
+    if (Store == kStoreF32) {
+      const float* s = static_cast<const float*>(a.src);
+      f[i] = s[e];
+      if (two) g[i] = s[e + a.ps];
+    } else {
+      const __nv_bfloat16* s = static_cast<const __nv_bfloat16*>(a.src);
+      f[i] = __bfloat162float(s[e]);
+      if (two) g[i] = __bfloat162float(s[e + a.ps]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    fm = fmaxf(fm, fabsf(f[i]));
+    gm = fmaxf(gm, fabsf(g[i]));
+  }
+  const PartUnits fu(fm), gu(gm);
+  Parts R[kQ1], C[kQ1], G;
 #pragma unroll
   for (int ia = 0; ia < kQ1; ++ia)
 #pragma unroll
     for (int ib = 0; ib < kQ1; ++ib) {
-      const size_t e = (size_t)(kQ1 * ia + ib) * a.plane_stride + o;
-      float f, g = 0.f;
-      if (Store == kStoreF32) {
-        const float* s = static_cast<const float*>(a.src);
-        f = s[e];
-        if (two) g = s[e + a.ps];
-      } else {
-        const __nv_bfloat16* s = static_cast<const __nv_bfloat16*>(a.src);
-        f = __bfloat162float(s[e]);
-        if (two) g = __bfloat162float(s[e + a.ps]);
-      }
-      two_sum(rh[ia], rl[ia], f);
-      two_sum(ch[ib], cl[ib], f);
-      two_sum(gh, gl, g);
+      const Parts x = fu.split(f[kQ1 * ia + ib]);
+      R[ia] = R[ia] + x;
+      C[ib] = C[ib] + x;
+      G = G + gu.split(g[kQ1 * ia + ib]);
     }
-  // (an infinite sum has no error term)
-  auto finite = [](float e) { return e == e ? e : 0.f; };
-  double R[kQ1], C[kQ1];
-#pragma unroll
-  for (int k = 0; k < kQ1; ++k) {
-    rl[k] = finite(rl[k]);
-    cl[k] = finite(cl[k]);
-    R[k] = exact_double(rh[k]) + exact_double(rl[k]);
-    C[k] = exact_double(ch[k]) + exact_double(cl[k]);
-  }
-  const double s = a.cs.xi[1], l = a.cs.xi[2], r13 = R[1] + R[3], r24 = R[2] + R[4];
-  *drho = R[0] + r13 + r24;
-  *jx = s * (R[1] - R[3]) + l * (R[2] - R[4]);
-  *jy = s * (C[1] - C[3]) + l * (C[2] - C[4]);
-  *e2 = s * s * (r13 + C[1] + C[3]) + l * l * (r24 + C[2] + C[4]) + (exact_double(gh) + exact_double(finite(gl)));
+  const Parts r13 = R[1] + R[3], r24 = R[2] + R[4];
+  const double s = a.cs.xi[1], l = a.cs.xi[2];
+  *drho = (R[0] + r13 + r24).value();
+  *jx = s * (R[1] - R[3]).value() + l * (R[2] - R[4]).value();
+  *jy = s * (C[1] - C[3]).value() + l * (C[2] - C[4]).value();
+  *e2 = s * s * (r13 + C[1] + C[3]).value() + l * l * (r24 + C[2] + C[4]).value() + G.value();
+  return fm < 0x1p120f && gm < 0x1p120f && isfinite(*drho) && isfinite(*e2);   // (fmaxf passes over NaN)
 }
 
 template <int Store, bool Q25>
@@ -75,8 +94,10 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(const __grid_const
     const int npop = a.cp.npop;
     double rho = 0.0, jx = 0.0, jy = 0.0, e2 = 0.0;
     const int nq1 = a.cs.nq1;
-    if constexpr (Q25) moments25<Store>(a, o, &rho, &jx, &jy, &e2);
-    for (int i = 0; i < (Q25 ? 0 : nq1 * nq1); ++i) {
+    bool summed = false;
+    if constexpr (Q25) summed = moments25<Store>(a, o, &rho, &jx, &jy, &e2);
+    if (Q25 && !summed) rho = jx = jy = e2 = 0.0;
+    for (int i = summed ? nq1 * nq1 : 0; i < nq1 * nq1; ++i) {
       const double cx = a.cs.xi[i / nq1], cy = a.cs.xi[i % nq1];
       double fv, gv = 0.0;
       if (Store == kStoreF64) {
