@@ -27,11 +27,13 @@ class SLLBMRollout(torch.autograd.Function):
             sim.init(rho0, u0, v0, T0)
             # a segment a call: get_state returns a tensor of its own, and small states replay the
             # step's graph within a call
-            checkpoints = {0: sim.get_state()}
-            for start in range(0, nsteps, k):
-                sim.step(min(k, nsteps - start))
-                if start + k < nsteps:
-                    checkpoints[start + k] = sim.get_state()
+            checkpoints, done = {0: sim.get_state()}, 0
+            for n in range(1, nsteps + 1):
+                if n % k == 0 or n == nsteps:
+                    sim.step(n - done)
+                    done = n
+                    if n < nsteps:
+                        checkpoints[n] = sim.get_state()
             rho = sim.moments(sums=False)["rho"].double()
         ctx.sim, ctx.nsteps, ctx.k, ctx.checkpoints = sim, nsteps, k, checkpoints
         ctx.save_for_backward(u0, v0, rho0, T0)
