@@ -396,78 +396,89 @@ cudaError_t launch_ghost_fill(void* origin, int elem, size_t plane_stride, int p
 // ------------------------------------------------------------------------------------------
 // Dense [npop][nq][ny][nx] <-> internal layout (ghost cells, row pitch, interleaved pairs).
 // ------------------------------------------------------------------------------------------
-// A block of 64 x 4 threads takes chunks of 256 columns of 4 rows, a thread 4 columns 64 apart: four
-// coalesced accesses a thread in flight (one a thread held the copies at 4.4 TB/s on 3073 x 3073 vertices,
-// and the index divisions of a flat layout at 1.6 TB/s on the D2Q9 state of 2048 x 2048).
-constexpr int kConvX = 64, kConvY = 4, kConvPer = 4;
+// A block of 256 threads takes bx x (256 / bx) of them, a thread 4 values: four coalesced accesses a thread in
+// flight (one a thread held the copies at 4.4 TB/s on 3073 x 3073 vertices, and the index divisions of a
+// flat layout at 1.6 TB/s on the D2Q9 state of 2048 x 2048).  Rows of more than 128 columns: bx = 64, the 4 values
+// 64 columns apart.  Shorter rows: bx the least power of two that holds one, the 4 values in rows 256 / bx apart,
+// so that at least half the threads have work
+// (with bx = 64 throughout 7 x 20000 vertices in FP64 took 261 us, now 75; 17 x 160000 in FP32 1.78 ms, now 0.52).
+constexpr int kConvThreads = 256, kConvPer = 4, kConvX = 64;
 
-static dim3 convert_grid(int nx, int ny, int planes) {
-  const int rows = (ny + kConvY - 1) / kConvY;
-  return dim3((unsigned)((nx + kConvX * kConvPer - 1) / (kConvX * kConvPer)), (unsigned)(rows < 65535 ? rows : 65535),
-              (unsigned)planes);
+struct ConvLayout {
+  dim3 grid, block;
+  bool wide;
+};
+
+static ConvLayout convert_layout(int nx, int ny, int planes) {
+  const bool wide = nx > 128;
+  int bx = wide ? kConvX : 1;
+  while (!wide && bx < nx) bx *= 2;
+  const int by = kConvThreads / bx, cols = wide ? bx * kConvPer : bx, per = wide ? by : by * kConvPer;   // a block's
+  const int rows = (ny + per - 1) / per;
+  return ConvLayout{dim3((unsigned)((nx + cols - 1) / cols), (unsigned)(rows < 65535 ? rows : 65535), (unsigned)planes),
+                    dim3((unsigned)bx, (unsigned)by), wide};
 }
 
-template <typename E>
-__global__ void __launch_bounds__(kConvX* kConvY)
+template <typename E, bool Wide>
+__global__ void __launch_bounds__(kConvThreads)
     state_convert_kernel(const E* src, E* dst, int to_internal, int plane0, int nq, int nx, int ny, int pitch,
                          size_t plane_stride, int xs, ptrdiff_t ps) {
-  const int x0 = blockIdx.x * (kConvX * kConvPer) + threadIdx.x, pl = plane0 + blockIdx.z;
-  const int pop = pl / nq, i = pl - pop * nq;
-  for (int y = blockIdx.y * kConvY + threadIdx.y; y < ny; y += gridDim.y * kConvY) {
-    const size_t d = ((size_t)pl * ny + y) * nx;                                                 // dense row
-    const ptrdiff_t o = (ptrdiff_t)(i * plane_stride) + pop * ps + (ptrdiff_t)y * pitch;      // internal row
+  const int pl = plane0 + blockIdx.z, pop = pl / nq, i = pl - pop * nq;
+  const int x = blockIdx.x * (Wide ? kConvPer * kConvX : blockDim.x) + threadIdx.x;
+  const int by = Wide ? kConvThreads / kConvX : blockDim.y, per = Wide ? by : kConvPer * by;   // rows a block
+  const int sd = Wide ? kConvX : by * nx, so = Wide ? kConvX * xs : by * pitch;               // to the next value
+  for (int y = blockIdx.y * per + threadIdx.y; y < ny; y += gridDim.y * per) {
+    const size_t d = ((size_t)pl * ny + y) * nx + x;                                                            // dense
+    const ptrdiff_t o = (ptrdiff_t)(i * plane_stride) + pop * ps + (ptrdiff_t)y * pitch + (ptrdiff_t)x * xs;   // internal
     E v[kConvPer];
 #pragma unroll
-    for (int k = 0; k < kConvPer; ++k) {
-      const int x = x0 + k * kConvX;
-      if (x < nx) v[k] = to_internal ? src[d + x] : src[o + (ptrdiff_t)x * xs];
-    }
+    for (int k = 0; k < kConvPer; ++k)
+      if (Wide ? x + k * kConvX < nx : x < nx && y + k * by < ny) v[k] = to_internal ? src[d + k * sd] : src[o + k * so];
 #pragma unroll
-    for (int k = 0; k < kConvPer; ++k) {
-      const int x = x0 + k * kConvX;
-      if (x < nx) {
+    for (int k = 0; k < kConvPer; ++k)
+      if (Wide ? x + k * kConvX < nx : x < nx && y + k * by < ny) {
         if (to_internal)
-          dst[o + (ptrdiff_t)x * xs] = v[k];
+          dst[o + k * so] = v[k];
         else
-          dst[d + x] = v[k];
+          dst[d + k * sd] = v[k];
       }
-    }
   }
 }
 
 // Dense [npop][nq][ny][nx] <-> interleaved (f, g) pairs (xs = 2, ps = 1) for the velocity planes
 // i0 .. i0 + gridDim.z - 1: f and g together, so that a pair moves as one 8-byte (FP32) or 4-byte
 // (BF16) access (g = 0 with one population).
-template <typename E, typename E2>
-__global__ void __launch_bounds__(kConvX* kConvY)
+template <typename E, typename E2, bool Wide>
+__global__ void __launch_bounds__(kConvThreads)
     pair_convert_kernel(const E* src, E* dst, int to_internal, int i0, int npop, int nq, int nx, int ny, int pitch,
                         size_t plane_stride) {
-  const int x0 = blockIdx.x * (kConvX * kConvPer) + threadIdx.x, i = i0 + blockIdx.z;
+  const int i = i0 + blockIdx.z;
+  const int x = blockIdx.x * (Wide ? kConvPer * kConvX : blockDim.x) + threadIdx.x;
+  const int by = Wide ? kConvThreads / kConvX : blockDim.y, per = Wide ? by : kConvPer * by;   // rows a block
+  const int sd = Wide ? kConvX : by * nx, so = Wide ? 2 * kConvX : by * pitch;                // to the next pair
   const size_t gd = (size_t)nq * nx * ny;   // from f to g in the dense layout
-  for (int y = blockIdx.y * kConvY + threadIdx.y; y < ny; y += gridDim.y * kConvY) {
-    const size_t d = ((size_t)i * ny + y) * nx;                         // f row in the dense layout
-    const size_t o = (size_t)i * plane_stride + (size_t)y * pitch;   // row of pairs
+  for (int y = blockIdx.y * per + threadIdx.y; y < ny; y += gridDim.y * per) {
+    const size_t d = ((size_t)i * ny + y) * nx + x;                                        // f in the dense layout
+    const size_t o = (size_t)i * plane_stride + (size_t)y * pitch + 2 * (size_t)x;       // the pair
     E2 p[kConvPer];
 #pragma unroll
     for (int k = 0; k < kConvPer; ++k) {
-      const int x = x0 + k * kConvX;
-      if (x >= nx) continue;
+      if (!(Wide ? x + k * kConvX < nx : x < nx && y + k * by < ny)) continue;
       if (to_internal) {
-        p[k].x = src[d + x];
-        p[k].y = npop == 2 ? src[gd + d + x] : E(0);
+        p[k].x = src[d + k * sd];
+        p[k].y = npop == 2 ? src[gd + d + k * sd] : E(0);
       } else {
-        p[k] = *reinterpret_cast<const E2*>(src + o + 2 * (size_t)x);
+        p[k] = *reinterpret_cast<const E2*>(src + o + k * so);
       }
     }
 #pragma unroll
     for (int k = 0; k < kConvPer; ++k) {
-      const int x = x0 + k * kConvX;
-      if (x >= nx) continue;
+      if (!(Wide ? x + k * kConvX < nx : x < nx && y + k * by < ny)) continue;
       if (to_internal) {
-        *reinterpret_cast<E2*>(dst + o + 2 * (size_t)x) = p[k];
+        *reinterpret_cast<E2*>(dst + o + k * so) = p[k];
       } else {
-        dst[d + x] = p[k].x;
-        if (npop == 2) dst[gd + d + x] = p[k].y;
+        dst[d + k * sd] = p[k].x;
+        if (npop == 2) dst[gd + d + k * sd] = p[k].y;
       }
     }
   }
@@ -477,14 +488,17 @@ cudaError_t launch_pair_convert(const void* src, void* dst, bool to_internal, in
                                 int nq, int nx, int ny, int pitch, size_t plane_stride, cudaStream_t s) {
   if (ni == 0) return cudaSuccess;
   if (ny > 65535 || ni > 65535) return cudaErrorInvalidValue;
-  const dim3 grid = convert_grid(nx, ny, ni), block(kConvX, kConvY);
+  const ConvLayout cl = convert_layout(nx, ny, ni);
   const int ti = to_internal ? 1 : 0;
+  auto launch = [&](auto* kern, auto e) {
+    using E = decltype(e);
+    kern<<<cl.grid, cl.block, 0, s>>>(static_cast<const E*>(src), static_cast<E*>(dst), ti, i0, npop, nq, nx, ny, pitch,
+                                      plane_stride);
+  };
   if (elem == 4)
-    pair_convert_kernel<uint32_t, uint2><<<grid, block, 0, s>>>(static_cast<const uint32_t*>(src),
-        static_cast<uint32_t*>(dst), ti, i0, npop, nq, nx, ny, pitch, plane_stride);
+    launch(cl.wide ? pair_convert_kernel<uint32_t, uint2, true> : pair_convert_kernel<uint32_t, uint2, false>, uint32_t{});
   else if (elem == 2)
-    pair_convert_kernel<uint16_t, ushort2><<<grid, block, 0, s>>>(static_cast<const uint16_t*>(src),
-        static_cast<uint16_t*>(dst), ti, i0, npop, nq, nx, ny, pitch, plane_stride);
+    launch(cl.wide ? pair_convert_kernel<uint16_t, ushort2, true> : pair_convert_kernel<uint16_t, ushort2, false>, uint16_t{});
   else
     return cudaErrorInvalidValue;
   return cudaGetLastError();
@@ -495,21 +509,17 @@ cudaError_t launch_state_convert(const void* src, void* dst, bool to_internal, i
                                  int xs, ptrdiff_t ps, cudaStream_t s) {
   if (nplanes == 0) return cudaSuccess;
   if (nplanes > 65535) return cudaErrorInvalidValue;
-  const dim3 blocks = convert_grid(nx, ny, nplanes), threads(kConvX, kConvY);
+  const ConvLayout cl = convert_layout(nx, ny, nplanes);
   const int ti = to_internal ? 1 : 0;
+  auto launch = [&](auto* kern, auto e) {
+    using E = decltype(e);
+    kern<<<cl.grid, cl.block, 0, s>>>(static_cast<const E*>(src), static_cast<E*>(dst), ti, plane0, nq, nx, ny, pitch,
+                                      plane_stride, xs, ps);
+  };
   switch (elem) {
-    case 2:
-      state_convert_kernel<uint16_t><<<blocks, threads, 0, s>>>(static_cast<const uint16_t*>(src),
-          static_cast<uint16_t*>(dst), ti, plane0, nq, nx, ny, pitch, plane_stride, xs, ps);
-      break;
-    case 4:
-      state_convert_kernel<uint32_t><<<blocks, threads, 0, s>>>(static_cast<const uint32_t*>(src),
-          static_cast<uint32_t*>(dst), ti, plane0, nq, nx, ny, pitch, plane_stride, xs, ps);
-      break;
-    case 8:
-      state_convert_kernel<uint64_t><<<blocks, threads, 0, s>>>(static_cast<const uint64_t*>(src),
-          static_cast<uint64_t*>(dst), ti, plane0, nq, nx, ny, pitch, plane_stride, xs, ps);
-      break;
+    case 2: launch(cl.wide ? state_convert_kernel<uint16_t, true> : state_convert_kernel<uint16_t, false>, uint16_t{}); break;
+    case 4: launch(cl.wide ? state_convert_kernel<uint32_t, true> : state_convert_kernel<uint32_t, false>, uint32_t{}); break;
+    case 8: launch(cl.wide ? state_convert_kernel<uint64_t, true> : state_convert_kernel<uint64_t, false>, uint64_t{}); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
