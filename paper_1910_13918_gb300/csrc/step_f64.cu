@@ -1,7 +1,7 @@
 // Plain FP64 SLLBM step on full populations: the accuracy and speed baseline of the FP32 paths.
 // Moments (Sec. II), the fourth-order equilibrium (Sec. II.A) and BGK (Eq. streaming_fg).
 //
-// step_tile_f64_kernel (uniform grids, Pr = 1): tiles of 32 x 4 vertices, sum factorisation through
+// step_tile_f64_kernel (uniform grids that fill its tiles, Pr = 1): tiles of 32 x 4 vertices, sum factorisation through
 // shared memory.  step_plain_f64_kernel (the rest): one thread per vertex, (p+1)^2 gathers per
 // velocity plane from global memory with FP64 weights.
 #include "kernels.h"
@@ -196,12 +196,28 @@ __global__ void __launch_bounds__(kFN, 3) step_tile_f64_kernel(const __grid_cons
   if (!(rho > 0.0 && theta > 0.0 && isfinite(rho) && isfinite(theta))) atomicOr(a.flag, 1);
 }
 
+// Whether the tiles are filled well enough: vertices past the grid cost as much as others, so on grids of
+// a few columns (or rows) the gathers are faster.  The lines are where the two cross on grids of 4,800 and
+// 24,000 rows (7 x 20000 vertices, p = 1: 306 us a step by gathers, 723 in tiles; 16 x 24000, p = 4: 1569 and 1228);
+// the gathers' longer start is worth some 12,000 vertices at p <= 2 (24000 x 5, p = 1: 263 and 210).
+// Tiles that are all resident at once (three blocks an SM) wait for latency, not for the pipe, and are the
+// shorter way at any filling (6 x 480, p = 1: 38 us and 60; 12 x 1820: 70 and 79; at p = 1 the third block of
+// fewer than 12 columns is not: 8 x 1820 69 and 55).
+bool tile_f64_pays(const StepArgs& a) {
+  const long long tiles = (long long)((a.nx + kFX - 1) / kFX) * ((a.ny + kFY - 1) / kFY);
+  int dev = 0, n_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return true;   // (the launch reports the error)
+  const double least[5] = {1.0, 0.65, 0.58, 0.49, 0.41};
+  return tiles <= (a.P == 1 && a.nx < 12 ? 2LL : 3LL) * n_sm || (double)a.nv + (a.P <= 2 ? 12400.0 : 0.0) >= least[a.P] * (double)(tiles * kFN);
+}
+
 // The tile kernel takes the step: a uniform grid, Pr = 1, and a window a block can stage.
 bool tile_f64_window(const StepArgs& a, F64Window* w) {
   if (a.mapped || a.cp.pr_on || a.cs.nq1 != kQ1) return false;
   *w = F64Window{a.offx_min, a.offy_min, kFX + a.offx_max - a.offx_min, kFY + a.offy_max - a.offy_min};
   // (the window holds each vertex itself: components at rest have offsets in [-p, 0] and ends in [0, p])
-  return w->ox <= 0 && w->oy <= 0 && a.offx_max >= 0 && a.offy_max >= 0 && w->W * w->H <= kFElems * kFN;
+  return w->ox <= 0 && w->oy <= 0 && a.offx_max >= 0 && a.offy_max >= 0 && w->W * w->H <= kFElems * kFN && tile_f64_pays(a);
 }
 
 }  // namespace
