@@ -22,6 +22,7 @@ constexpr int kXferChunks = 5;   // host transfers move the state in this many p
 // direct launches are as fast.)
 constexpr int kGraphMinSteps = 4;
 constexpr size_t kGraphMaxStateBytes = size_t(64) << 20;
+constexpr long long kFixMaxVertices = 2000;   // more off the cell pattern go to edge tiles (build_uniform_pattern)
 
 struct sllbm_ctx {
   sllbm_grid_desc g;
@@ -381,10 +382,13 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c) {
   // Vertices off the pattern, next to zero-gradient boundaries.  On states beyond the L2 a second
   // launch of the fused kernel does the tiles that hold them: gathered one by one from HBM, each
   // of the 25 planes of a boundary column touches pages of its own (3073^2 vertices, p = 3: 0.857 ms
-  // a step so, 0.905 ms with the fix-up kernel).  On states in the L2 the fix-up kernel's single
-  // gather per warp is the shorter one (8193 x 8, p = 2: 17.5 us a step, 18.4 us with edge tiles).
+  // a step so, 0.905 ms with the fix-up kernel).  On states in the L2 it is a matter of how many they are: a few
+  // take one gather a warp beside the last tiles (8193 x 8 with ends, 16 vertices: 12.5 us a step, 13.7 with
+  // edge tiles; 201^2, 800: 11.5 and 13.5), thousands come in waves after them (9 x 8193, 16,400, p = 2:
+  // 35.8 and 18.4; 13 x 8193, p = 4: 61.7 and 19.7; between 1,000 and 2,000 either may be the faster).
   const bool uneven = px.lo > 0 || px.hi < c->nx || py.lo > 0 || py.hi < c->ny;
-  c->ut.edge = uneven && px.whole && py.whole && dense_bytes(c) > kGraphMaxStateBytes;
+  const long long n_off = c->nv - (long long)std::count(sx.begin(), sx.end(), 1) * std::count(sy.begin(), sy.end(), 1);
+  c->ut.edge = uneven && px.whole && py.whole && (dense_bytes(c) > kGraphMaxStateBytes || n_off > kFixMaxVertices);
   if (c->ut.edge) {
     if (!c->etail[0]) {
       TRY(dalloc(c, &c->etail[0], px.tail.size()));
