@@ -272,29 +272,28 @@ static GeomArgs geom_args(sllbm_ctx* c) {
   return g;
 }
 
-// Cell-periodic pattern of the per-axis tables of a uniform grid (read by step_uniform.cu):
-// taken from a cell in the middle of each axis; a vertex "follows the pattern" when its offset
-// and weights match those of its local node for all five components.  The fused kernel writes
-// only vertices that follow the pattern on both axes; the others go to the gather kernel.
-// Every vertex's own stencil is kept too, as the fused kernel's edge tiles read it: tail sums of the
-// weights and whether it is the cell before the vertex's own (whole: all stencils are one of the
-// two).
+// Cell-periodic pattern of the per-axis tables of a uniform grid (read by step_uniform.cuh and the
+// whole-cell kernel of step_q9.cu): taken from a cell in the middle of each axis; a vertex "follows the
+// pattern" when its offset and weights match those of its local node for all components.  The
+// others go to the fix-up kernel or the edge tiles of the fused kernel (whole: all stencils are the
+// vertex's own cell or the one before it, as the edge tiles take them).
 struct AxisPattern {
+  explicit AxisPattern(const std::vector<int>& o) : off(o) {}
+  const std::vector<int>& off;          // [components][n]: the axis table
+  std::vector<double> w;                // [components][n][p + 1]
   std::vector<unsigned char> follows;   // [n]
-  std::vector<float4> tail;             // [5][n]: W_1..W_P, W_alpha = sum_{beta >= alpha} w_beta
-  std::vector<unsigned char> before;    // [5][n]
   bool whole = true;
   int lo = 0, hi = 0;                   // the run of vertices around the middle that follow the pattern
 };
 
-static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const int* off_dev, const double* w_dev,
-                                 bool is_y, AxisPattern& pat, bool* ok) {
+static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const double* w_dev, bool is_y, AxisPattern& pat,
+                                 bool* ok) {
   std::vector<unsigned char>& stdv = pat.follows;
   const int n = ax.nv, P = c->P;
   const int nq1 = c->nq1;
-  std::vector<int> off((size_t)nq1 * n);
-  std::vector<double> w((size_t)nq1 * n * (P + 1));
-  CUDA_TRY(c, cudaMemcpyAsync(off.data(), off_dev, off.size() * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  const std::vector<int>& off = pat.off;
+  std::vector<double>& w = pat.w;
+  w.resize((size_t)nq1 * n * (P + 1));
   CUDA_TRY(c, cudaMemcpyAsync(w.data(), w_dev, w.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   *ok = ax.n_cells >= 3;
@@ -326,20 +325,10 @@ static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const int* off_d
       if (!same) stdv[j] = 0;
     }
   }
-  pat.tail.resize((size_t)nq1 * n);
-  pat.before.resize((size_t)nq1 * n);
-  for (int comp = 0; comp < nq1; ++comp)
-    for (int j = 0; j < n; ++j) {
-      const size_t e = (size_t)comp * n + j;
-      float tail[4] = {0.f, 0.f, 0.f, 0.f};
-      double acc = 0.0;
-      for (int al = P; al >= 1; --al) {
-        acc += w[e * (P + 1) + al];
-        tail[al - 1] = (float)acc;
-      }
-      pat.tail[e] = make_float4(tail[0], tail[1], tail[2], tail[3]);
-      pat.before[e] = j % P == 0 && off[e] == -P;
-      if (!pat.before[e] && off[e] != -(j % P)) pat.whole = false;
+  for (int comp = 0; comp < nq1 && pat.whole; ++comp)
+    for (int j = 0; j < n && pat.whole; ++j) {
+      const int d = off[(size_t)comp * n + j], l = j % P;
+      pat.whole = d == -l || (l == 0 && d == -P);
     }
   pat.lo = pat.hi = jref0;
   while (pat.lo > 0 && stdv[pat.lo - 1]) --pat.lo;
@@ -347,18 +336,36 @@ static sllbm_status axis_pattern(sllbm_ctx* c, const AxisK& ax, const int* off_d
   return SLLBM_OK;
 }
 
-static sllbm_status build_uniform_pattern(sllbm_ctx* c) {
+// Every vertex's own stencil, as the edge tiles of the fused kernel read it: tail sums of the weights
+// (W_1..W_P, W_alpha = sum_{beta >= alpha} w_beta) and whether it is the cell before, [5][n] each.
+static void edge_tables(const AxisPattern& pat, int n, int P, std::vector<float4>& tail, std::vector<unsigned char>& before) {
+  tail.resize(pat.off.size());
+  before.resize(pat.off.size());
+  for (size_t e = 0; e < tail.size(); ++e) {
+    float t[4] = {0.f, 0.f, 0.f, 0.f};
+    double acc = 0.0;
+    for (int al = P; al >= 1; --al) {
+      acc += pat.w[e * (P + 1) + al];
+      t[al - 1] = (float)acc;
+    }
+    tail[e] = make_float4(t[0], t[1], t[2], t[3]);
+    before[e] = (int)(e % n) % P == 0 && pat.off[e] == -P;
+  }
+}
+
+// ox, oy: the offset tables of the axes.
+static sllbm_status build_uniform_pattern(sllbm_ctx* c, const std::vector<int>& ox, const std::vector<int>& oy) {
   c->ut.valid = false;
   // Any vertex count: the tensor copies start on 16-byte boundaries of the padded rows whatever nx
   // is, and the ghost cells carry the periodic seam.  (Periodic axes of nx % 4 != 0 took the gather
   // kernel before: 1.13 ms a step on 1023 x 1023 vertices of order 3, 0.106 ms here.)
   const bool q9 = c->nq1 == 3;
   if (c->xs != 2 && !(q9 && c->store != kStoreF64)) return SLLBM_OK;
-  AxisPattern px, py;
+  AxisPattern px(ox), py(oy);
   const std::vector<unsigned char>&sx = px.follows, &sy = py.follows;
   bool okx = false, oky = false;
-  TRY(axis_pattern(c, c->ax, c->offx, c->wx64, false, px, &okx));
-  TRY(axis_pattern(c, c->ay, c->offy, c->wy64, true, py, &oky));
+  TRY(axis_pattern(c, c->ax, c->wx64, false, px, &okx));
+  TRY(axis_pattern(c, c->ay, c->wy64, true, py, &oky));
   if (!okx || !oky) return SLLBM_OK;
   // The fused kernel takes each stencil as a whole cell, on both axes: start offset -l at local
   // node l, or -P at node 0 (a departure into the cell before).  Anything else goes to the
@@ -390,16 +397,14 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c) {
   const long long n_off = c->nv - (long long)std::count(sx.begin(), sx.end(), 1) * std::count(sy.begin(), sy.end(), 1);
   c->ut.edge = uneven && px.whole && py.whole && (dense_bytes(c) > kGraphMaxStateBytes || n_off > kFixMaxVertices);
   if (c->ut.edge) {
-    if (!c->etail[0]) {
-      TRY(dalloc(c, &c->etail[0], px.tail.size()));
-      TRY(dalloc(c, &c->etail[1], py.tail.size()));
-      TRY(dalloc(c, &c->ebef[0], px.before.size()));
-      TRY(dalloc(c, &c->ebef[1], py.before.size()));
-    }
     for (int k = 0; k < 2; ++k) {
-      const AxisPattern& pat = k ? py : px;
-      CUDA_TRY(c, cudaMemcpy(c->etail[k], pat.tail.data(), pat.tail.size() * sizeof(float4), cudaMemcpyHostToDevice));
-      CUDA_TRY(c, cudaMemcpy(c->ebef[k], pat.before.data(), pat.before.size(), cudaMemcpyHostToDevice));
+      std::vector<float4> tail;
+      std::vector<unsigned char> before;
+      edge_tables(k ? py : px, k ? c->ny : c->nx, c->P, tail, before);
+      if (!c->etail[k]) TRY(dalloc(c, &c->etail[k], tail.size()));
+      if (!c->ebef[k]) TRY(dalloc(c, &c->ebef[k], before.size()));
+      CUDA_TRY(c, cudaMemcpy(c->etail[k], tail.data(), tail.size() * sizeof(float4), cudaMemcpyHostToDevice));
+      CUDA_TRY(c, cudaMemcpy(c->ebef[k], before.data(), before.size(), cudaMemcpyHostToDevice));
     }
     c->ut.tail_x = c->etail[0];
     c->ut.tail_y = c->etail[1];
@@ -856,6 +861,7 @@ sllbm_status sllbm_precompute_departures(sllbm_ctx* c) {
   if (!c) return SLLBM_ERR_ARG;
   GeomArgs g = geom_args(c);
   const bool mapped = c->map.kind != SLLBM_MAP_IDENTITY;
+  std::vector<int> ox, oy;
   if (!mapped) {  // per-axis tables
     if (!c->offx) {
       TRY(dalloc(c, &c->offx, kQ1 * (size_t)c->nx));
@@ -867,7 +873,8 @@ sllbm_status sllbm_precompute_departures(sllbm_ctx* c) {
     }
     CUDA_TRY(c, launch_axis_tables(c->ax, c->cs, c->p.dt, c->offx, c->wx, c->wx64, c->stream));
     CUDA_TRY(c, launch_axis_tables(c->ay, c->cs, c->p.dt, c->offy, c->wy, c->wy64, c->stream));
-    std::vector<int> ox(c->nq1 * (size_t)c->nx), oy(c->nq1 * (size_t)c->ny);
+    ox.resize(c->nq1 * (size_t)c->nx);
+    oy.resize(c->nq1 * (size_t)c->ny);
     CUDA_TRY(c, cudaMemcpyAsync(ox.data(), c->offx, ox.size() * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(oy.data(), c->offy, oy.size() * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -882,7 +889,7 @@ sllbm_status sllbm_precompute_departures(sllbm_ctx* c) {
   } else if (c->store == kStoreF64) {
     c->kernel = kKernelPlainF64;
   } else if (!mapped) {
-    TRY(build_uniform_pattern(c));
+    TRY(build_uniform_pattern(c, ox, oy));
     c->kernel = c->ut.valid ? kKernelUniform : kKernelGather;
   } else {
     c->kernel = kKernelGather;
@@ -908,7 +915,7 @@ sllbm_status sllbm_precompute_departures(sllbm_ctx* c) {
   if (c->kernel == kKernelQ9 && (c->store == kStoreF32 || c->store == kStoreBF16) && !mapped) {
     StepArgs a = step_args(c, c->state[0], c->state[1]);
     a.mapped = 0;
-    TRY(build_uniform_pattern(c));
+    TRY(build_uniform_pattern(c, ox, oy));
     c->q9_tma = !c->ut.valid && q9_tma_usable(a, c->elem) ? 1 : 0;
   }
   c->ghost.on = (c->kernel == kKernelUniform || c->kernel == kKernelMapped || c->q9_tma ||
