@@ -389,7 +389,8 @@ __global__ void __launch_bounds__(128, BLOCKS) step3d_f32_kernel(const __grid_co
 // pass a thread takes two neighbouring vertices: their common window comes in 16-byte loads, and
 // the two results leave in one 16-byte store.  The thread sums its vertices' moments over the 125
 // planes.  collide3d_kernel then relaxes every vertex's 125 pairs in place and writes the periodic
-// images of the vertices next to periodic faces.
+// images of the vertices next to periodic faces.  On grids of few tiles five CTAs share a tile's planes
+// (stream3d_parts).
 //
 // What bounds it: the latency of the phases and shared memory together (64^3: the LSU pipe at 65 %,
 // issue at 39 %; 128^3: 1.187 ms, 1.38 ms with three barriers a plane and one vertex a task).  Deeper
@@ -433,7 +434,7 @@ struct Stream3Args {
   const float2* src;     // pairs in layout lay (deviations)
   float2* dst;
   Pad3 lay;
-  float* sums;           // [6][nv]: sum f, sum f xi_x, sum f xi_y, sum f xi_z, sum f |xi|^2, sum g
+  float* sums;           // [parts][6][nv]: sum f, sum f xi_x, sum f xi_y, sum f xi_z, sum f |xi|^2, sum g
   int nx, ny, nz;
   long long nv;
   const float* tx;       // [5][nx][2p] tail sums per (component, node)
@@ -455,7 +456,8 @@ __device__ __forceinline__ float2 tail_interp(const float2 (&v)[N], const float2
   return acc;
 }
 
-template <int P>
+// NPL: the planes of a CTA, 125 or those of the x component blockIdx.y (25).
+template <int P, int NPL>
 __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
     stream3d_kernel(const __grid_constant__ Stream3Args a, const __grid_constant__ CUtensorMap smap) {
   using SH = T3Shape<P>;
@@ -471,7 +473,7 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
   uint64_t* BAR = reinterpret_cast<uint64_t*>(Wx + kQ1 * kT3X * NW);   // [NS]
   const int tid = threadIdx.x;
   const int tiles_x = (a.nx + kT3X - 1) / kT3X, tiles_y = (a.ny + kT3Y - 1) / kT3Y;
-  const int byz = (int)blockIdx.x / tiles_x;
+  const int byz = (int)blockIdx.x / tiles_x, first = NPL * (int)blockIdx.y;   // this CTA's planes
   const int x0 = ((int)blockIdx.x - byz * tiles_x) * kT3X, y0 = (byz % tiles_y) * kT3Y,
             z0 = (byz / tiles_y) * TZ;
   // the tile's tail sums of all components (nodes past the grid clamped: those outputs are not
@@ -499,10 +501,10 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
   // region origin in the ghost-padded layout (g = XO): x0 (x in floats: 2 x0, a multiple of 4, i.e.
   // 16 bytes), y0 - p + g, z0 - p + g
   const int cx = 2 * (x0 - XO + a.lay.g), cy = y0 - P + a.lay.g, cz = z0 - P + a.lay.g;
-  auto issue = [&](int i, int st) {   // thread 0: plane i into stage st
+  auto issue = [&](int i, int st) {   // thread 0: this CTA's plane i into stage st
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     mbar_expect_tx(&BAR[st], (unsigned)SH::kStage);
-    tma_load_4d(base + (size_t)st * SH::kStride, &smap, cx, cy, cz, i, &BAR[st]);
+    tma_load_4d(base + (size_t)st * SH::kStride, &smap, cx, cy, cz, first + i, &BAR[st]);
   };
   if (tid == 0)
     for (int k = 0; k < NS - 1; ++k) issue(k, k);
@@ -520,7 +522,7 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
   for (int k = 0; k < XT; ++k) {
     const int row = (tid + k * NT) >> 4, vy = y0 + row % kT3Y, vz = z0 + row / kT3Y;
     on[k] = vx < a.nx && vy < a.ny && vz < a.nz;
-    out[k] = a.dst + a.lay.at(0, vx, vy, vz);
+    out[k] = a.dst + a.lay.at(first, vx, vy, vz);
   }
   const bool both = vx + 1 < a.nx;   // an odd x count ends with half a task
   // per vertex: (sum f, sum g), sum f xi_y, sum f xi_z, sum f (xi_y^2 + xi_z^2); over the planes of
@@ -537,13 +539,13 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
   float wx[2][NW];
   int st = 0, par = 0;          // stage of plane i and the parity of its phase
   int zc = 0, yb = 0, yc = 0;   // component of the z pass (plane i); of the y pass (plane i - 1)
-  int xa = 0, xb = 0, xc = 0;   // components of the x pass (plane i - 2)
+  int xa = first / 25, xb = 0, xc = 0;   // components of the x pass (plane i - 2)
 #pragma unroll 1
-  for (int i = 0; i < kQ3 + 2; ++i) {
-    const bool late = i < kQ3 && !mbar_wait(&BAR[st], (unsigned)par, a.flag);
+  for (int i = 0; i < NPL + 2; ++i) {
+    const bool late = i < NPL && !mbar_wait(&BAR[st], (unsigned)par, a.flag);
     if (__syncthreads_or(late)) {
       // the copy of plane i did not land in time: stop, after it and the ones issued behind it
-      for (int k = i, s2 = st, p2 = par; k < i + NS - 1 && k < kQ3; ++k) {
+      for (int k = i, s2 = st, p2 = par; k < i + NS - 1 && k < NPL; ++k) {
         if (!mbar_wait(&BAR[s2], (unsigned)p2, a.flag)) break;
         if (++s2 == NS) {
           s2 = 0;
@@ -552,9 +554,9 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
       }
       return;
     }
-    if (tid == 0 && i + NS - 1 < kQ3) issue(i + NS - 1, st == 0 ? NS - 1 : st - 1);   // every thread is past plane i - 1
+    if (tid == 0 && i + NS - 1 < NPL) issue(i + NS - 1, st == 0 ? NS - 1 : st - 1);   // every thread is past plane i - 1
     // z pass of plane i: column (ry, rx) of the region, the tile's z rows
-    if (i < kQ3) {
+    if (i < NPL) {
       constexpr int ZR = (SH::ZT + NT - 1) / NT;
       const float2* Sst = reinterpret_cast<const float2*>(base + (size_t)st * SH::kStride);
       float2* zout = Zb + (i & 1) * SH::ZB;
@@ -586,7 +588,7 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
       if (++zc == kQ1) zc = 0;
     }
     // y pass of plane i - 1: column (tz, rx), the tile's y rows
-    if (i >= 1 && i <= kQ3) {
+    if (i >= 1 && i <= NPL) {
       if (yt >= 0) {
         const float* wy = Wy + yb * kT3Y * NW;
         const float2* zin = Zb + ((i - 1) & 1) * SH::ZB + ytz * SH::ZS + ycol;
@@ -687,7 +689,7 @@ __global__ void __launch_bounds__(T3Config<P>::NT, T3Config<P>::MINB)
       if (v2 == 1 && !both) continue;
       const float m[6] = {fg[k][v2].x, mx[k][v2], my[k][v2], mz[k][v2], m2[k][v2], fg[k][v2].y};
 #pragma unroll
-      for (int q = 0; q < 6; ++q) a.sums[(size_t)q * a.nv + v + v2] = m[q];
+      for (int q = 0; q < 6; ++q) a.sums[(size_t)(6 * blockIdx.y + q) * a.nv + v + v2] = m[q];
     }
   }
 }
@@ -703,6 +705,7 @@ struct Collide3Args {
   float2* dst;
   Pad3 lay;
   const float* sums;
+  int parts;             // of the moment sums
   int nx, ny, nz, px, py, pz;
   long long nv;
   Consts cs;
@@ -755,9 +758,13 @@ __global__ void __launch_bounds__(128, 5) collide3d_kernel(const __grid_constant
 #pragma unroll
   for (int ic = 0; ic < kQ1; ++ic) nxt[ic] = *at(kQ1 + ic);
   const size_t sp = (size_t)a.nv;
-  const float drho = a.sums[v], jx = a.sums[sp + v], jy = a.sums[2 * sp + v], jz = a.sums[3 * sp + v],
-              a2 = a.sums[4 * sp + v];
-  const float G = a.npop == 2 ? a.sums[5 * sp + v] : 0.f;
+  float mom[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) mom[q] = a.sums[q * sp + v];
+  for (int k = 1; k < a.parts; ++k)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) mom[q] += a.sums[(6 * k + q) * sp + v];
+  const float drho = mom[0], jx = mom[1], jy = mom[2], jz = mom[3], a2 = mom[4], G = a.npop == 2 ? mom[5] : 0.f;
   const float rho = 1.f + drho, inv_rho = __frcp_rn(rho);
   const float ux = jx * inv_rho, uy = jy * inv_rho, uz = jz * inv_rho;
   const float qk = (a2 + G - rho * (ux * ux + uy * uy + uz * uz) - 2.f * a.cv * drho) * inv_rho * a.inv2cv;
@@ -1117,7 +1124,8 @@ struct sllbm3d_ctx {
   bool tiled = false;
   Pad3 lay{};                            // layout of the FP32 pair state
   float* tail[3] = {nullptr, nullptr, nullptr};
-  float* sums = nullptr;
+  float* sums = nullptr;                 // [parts][6][nv]
+  int parts = 1;                         // CTAs a tile in stream3d_kernel, an x component each, or one
   int* flag = nullptr;
   std::vector<void*> allocations;
   std::string err;
@@ -1156,9 +1164,14 @@ size_t state_doubles(const sllbm3d_ctx* c) {
 }
 float2* pairs(const sllbm3d_ctx* c, int k) { return reinterpret_cast<float2*>(c->state[k]); }
 
-// The sum-factorised FP32 step: stream3d_kernel (a CTA per tile) then collide3d_kernel.
 template <int P>
-cudaError_t launch_stream3d(const Stream3Args& a, cudaStream_t s) {
+long long tiles3d(int nx, int ny, int nz) {
+  return (long long)((nx + kT3X - 1) / kT3X) * ((ny + kT3Y - 1) / kT3Y) * ((nz + T3Config<P>::TZ - 1) / T3Config<P>::TZ);
+}
+
+// The sum-factorised FP32 step: stream3d_kernel then collide3d_kernel.
+template <int P, int NPL>
+cudaError_t launch_stream3d_planes(const Stream3Args& a, cudaStream_t s) {
   using SH = T3Shape<P>;
   EncodeTiledFn enc = encode_fn();
   if (!enc) return cudaErrorNotSupported;
@@ -1176,11 +1189,34 @@ cudaError_t launch_stream3d(const Stream3Args& a, cudaStream_t s) {
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(stream3d_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::kBytes);
+  cudaError_t e = cudaFuncSetAttribute(stream3d_kernel<P, NPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::kBytes);
   if (e != cudaSuccess) return e;
-  const long long tiles = (long long)((a.nx + kT3X - 1) / kT3X) * ((a.ny + kT3Y - 1) / kT3Y) * ((a.nz + SH::TZ - 1) / SH::TZ);
-  stream3d_kernel<P><<<(unsigned)tiles, SH::NT, SH::kBytes, s>>>(a, smap);
+  stream3d_kernel<P, NPL><<<dim3((unsigned)tiles3d<P>(a.nx, a.ny, a.nz), kQ3 / NPL), SH::NT, SH::kBytes, s>>>(a, smap);
   return cudaGetLastError();
+}
+
+template <int P>
+cudaError_t launch_stream3d(const Stream3Args& a, int parts, cudaStream_t s) {
+  return parts == kQ1 ? launch_stream3d_planes<P, kQ3 / kQ1>(a, s) : launch_stream3d_planes<P, kQ3>(a, s);
+}
+
+// Whether a tile's 125 planes go to five CTAs, an x component each (with moment sums of their own), or to one.
+// A CTA runs one phase a plane and two more, at about 1 us each whatever the load: 127 phases a wave of
+// tiles, or 27 a wave of parts, which is what grids of a few tiles wait for (36 x 12 x 8, p = 1: 129 -> 50 us a step,
+// and 83 by the gather step; 49^3, p = 2: 230 -> 175; 64 x 32 x 32, p = 4: 216 -> 157).  Not where the tiles
+// fill the device as they are (64^3, p = 2, 256 tiles on 304 places: 298, 311 in parts) or beyond two
+// waves (128^3: 2.12 and 2.23 ms).
+int stream3d_parts(const sllbm3d_ctx* c) {
+  const int nx = c->ax.nv, ny = c->ay.nv, nz = c->az.nv;
+  long long tiles = 0, places = c->n_sm;
+  switch (c->g.order) {
+    case 1: tiles = tiles3d<1>(nx, ny, nz); places *= T3Config<1>::MINB; break;
+    case 2: tiles = tiles3d<2>(nx, ny, nz); places *= T3Config<2>::MINB; break;
+    case 3: tiles = tiles3d<3>(nx, ny, nz); places *= T3Config<3>::MINB; break;
+    default: tiles = tiles3d<4>(nx, ny, nz); places *= T3Config<4>::MINB; break;
+  }
+  auto waves = [&](long long n) { return (n + places - 1) / places; };
+  return places > 0 && tiles <= 2 * places && (kQ3 / kQ1 + 2) * waves(kQ1 * tiles) < (kQ3 + 2) * waves(tiles) ? kQ1 : 1;
 }
 
 // Whether the sum-factorised step takes the grid: FP32, axes at least as long as a staged region of
@@ -1215,7 +1251,8 @@ sllbm_status alloc_state3d(sllbm3d_ctx* c) {
   sllbm_status s = SLLBM_OK;
   for (int k = 0; k < 2 && s == SLLBM_OK; ++k) s = alloc3(c, &c->state[k], state_doubles(c));
   if (!c->tiled) return s;
-  if (s == SLLBM_OK) s = alloc3(c, &c->sums, (size_t)6 * c->nv);
+  c->parts = stream3d_parts(c);
+  if (s == SLLBM_OK) s = alloc3(c, &c->sums, (size_t)6 * c->parts * c->nv);
   for (int k = 0; k < 2 && s == SLLBM_OK; ++k)   // ghosts of zero-gradient faces stay 0
     s = cuda3(c, cudaMemsetAsync(c->state[k], 0, state_doubles(c) * sizeof(double), c->stream), "cudaMemsetAsync");
   return s;
@@ -1247,16 +1284,17 @@ cudaError_t launch_tiled3d(sllbm3d_ctx* c, const float2* src, float2* dst) {
   a.flag = c->flag;
   cudaError_t e = cudaErrorInvalidValue;
   switch (c->g.order) {
-    case 1: e = launch_stream3d<1>(a, c->stream); break;
-    case 2: e = launch_stream3d<2>(a, c->stream); break;
-    case 3: e = launch_stream3d<3>(a, c->stream); break;
-    case 4: e = launch_stream3d<4>(a, c->stream); break;
+    case 1: e = launch_stream3d<1>(a, c->parts, c->stream); break;
+    case 2: e = launch_stream3d<2>(a, c->parts, c->stream); break;
+    case 3: e = launch_stream3d<3>(a, c->parts, c->stream); break;
+    case 4: e = launch_stream3d<4>(a, c->parts, c->stream); break;
   }
   if (e != cudaSuccess) return e;
   Collide3Args b{};
   b.dst = dst;
   b.lay = c->lay;
   b.sums = c->sums;
+  b.parts = c->parts;
   b.nx = c->ax.nv;
   b.ny = c->ay.nv;
   b.nz = c->az.nv;
