@@ -272,6 +272,10 @@ static GeomArgs geom_args(sllbm_ctx* c) {
   return g;
 }
 
+// Tables are copied to the device in the order of the context's stream, which need not be ordered with the
+// default stream: a plain copy from pageable memory may return before its transfer has ended.  (The
+// asynchronous one returns when the host memory may be reused.)
+
 // Cell-periodic pattern of the per-axis tables of a uniform grid (read by step_uniform.cuh and the
 // whole-cell kernel of step_q9.cu): taken from a cell in the middle of each axis; a vertex "follows the
 // pattern" when its offset and weights match those of its local node for all components.  The
@@ -384,8 +388,8 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c, const std::vector<int>& 
     TRY(dalloc(c, &c->std_x, (size_t)c->nx));
     TRY(dalloc(c, &c->std_y, (size_t)c->ny));
   }
-  CUDA_TRY(c, cudaMemcpy(c->std_x, sx.data(), sx.size(), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(c->std_y, sy.data(), sy.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(c->std_x, sx.data(), sx.size(), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(c->std_y, sy.data(), sy.size(), cudaMemcpyHostToDevice, c->stream));
   // Vertices off the pattern, next to zero-gradient boundaries.  On states beyond the L2 a second
   // launch of the fused kernel does the tiles that hold them: gathered one by one from HBM, each
   // of the 25 planes of a boundary column touches pages of its own (3073^2 vertices, p = 3: 0.857 ms
@@ -403,8 +407,8 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c, const std::vector<int>& 
       edge_tables(k ? py : px, k ? c->ny : c->nx, c->P, tail, before);
       if (!c->etail[k]) TRY(dalloc(c, &c->etail[k], tail.size()));
       if (!c->ebef[k]) TRY(dalloc(c, &c->ebef[k], before.size()));
-      CUDA_TRY(c, cudaMemcpy(c->etail[k], tail.data(), tail.size() * sizeof(float4), cudaMemcpyHostToDevice));
-      CUDA_TRY(c, cudaMemcpy(c->ebef[k], before.data(), before.size(), cudaMemcpyHostToDevice));
+      CUDA_TRY(c, cudaMemcpyAsync(c->etail[k], tail.data(), tail.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream));
+      CUDA_TRY(c, cudaMemcpyAsync(c->ebef[k], before.data(), before.size(), cudaMemcpyHostToDevice, c->stream));
     }
     c->ut.tail_x = c->etail[0];
     c->ut.tail_y = c->etail[1];
@@ -417,7 +421,7 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c, const std::vector<int>& 
     std::vector<int2> tiles;
     uniform_edge_tiles(c->P, c->nx, c->ny, c->ut, tiles);
     if (!c->edge_tiles) TRY(dalloc(c, &c->edge_tiles, tiles.size()));
-    CUDA_TRY(c, cudaMemcpy(c->edge_tiles, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(c->edge_tiles, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice, c->stream));
     c->ut.edge_tiles = c->edge_tiles;
   }
   std::vector<int> fix;
@@ -428,7 +432,7 @@ static sllbm_status build_uniform_pattern(sllbm_ctx* c, const std::vector<int>& 
   c->n_fix = (long long)fix.size();
   if (!fix.empty()) {
     TRY(dalloc(c, &c->fix_list, fix.size()));
-    CUDA_TRY(c, cudaMemcpy(c->fix_list, fix.data(), fix.size() * sizeof(int), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(c->fix_list, fix.data(), fix.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   }
   c->ut.std_x = c->std_x;
   c->ut.std_y = c->std_y;
@@ -565,13 +569,13 @@ static sllbm_status build_mapped_tiles(sllbm_ctx* c) {
     TRY(dalloc(c, &c->morg, org.size()));
     TRY(dalloc(c, &c->mok, (size_t)ntiles));
   }
-  CUDA_TRY(c, cudaMemcpy(c->mrec, rec.data(), rec.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(c->morg, org.data(), org.size() * sizeof(int2), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(c->mok, ok.data(), ok.size(), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(c->mrec, rec.data(), rec.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(c->morg, org.data(), org.size() * sizeof(int2), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(c->mok, ok.data(), ok.size(), cudaMemcpyHostToDevice, c->stream));
   c->n_fix = (long long)fix.size();
   if (!fix.empty()) {
     TRY(dalloc(c, &c->fix_list, fix.size()));
-    CUDA_TRY(c, cudaMemcpy(c->fix_list, fix.data(), fix.size() * sizeof(int), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMemcpyAsync(c->fix_list, fix.data(), fix.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   }
   c->mt.rec = c->mrec;
   c->mt.dpitch = dpitch;
@@ -1183,9 +1187,9 @@ static sllbm_status upload_transpose(sllbm_ctx* c, const AxisTranspose& t, int n
   TRY(dalloc(c, col_dev, col.size()));
   TRY(dalloc(c, w_dev, wt.size()));
   TRY(dalloc(c, deg_dev, deg.size()));
-  CUDA_TRY(c, cudaMemcpy(*col_dev, col.data(), col.size() * sizeof(int), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(*w_dev, wt.data(), wt.size() * sizeof(float), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(*deg_dev, deg.data(), deg.size() * sizeof(int), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(*col_dev, col.data(), col.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(*w_dev, wt.data(), wt.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(*deg_dev, deg.data(), deg.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   return SLLBM_OK;
 }
 
@@ -1206,7 +1210,7 @@ static sllbm_status upload_dense_transpose(sllbm_ctx* c, const AxisTranspose& t,
       dense[r * dw + (d + h)] += e.second;
     }
   TRY(dalloc(c, dense_dev, dense.size()));
-  CUDA_TRY(c, cudaMemcpy(*dense_dev, dense.data(), dense.size() * sizeof(float), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(*dense_dev, dense.data(), dense.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
   return SLLBM_OK;
 }
 
@@ -1270,8 +1274,8 @@ static sllbm_status build_mapped_transpose(sllbm_ctx* c) {
     }
   TRY(dalloc(c, &c->tm_ptr, ptr.size()));
   TRY(dalloc(c, &c->tm_ent, (size_t)total));
-  CUDA_TRY(c, cudaMemcpy(c->tm_ptr, ptr.data(), ptr.size() * sizeof(long long), cudaMemcpyHostToDevice));
-  CUDA_TRY(c, cudaMemcpy(c->tm_ent, ent.data(), (size_t)total * sizeof(int2), cudaMemcpyHostToDevice));
+  CUDA_TRY(c, cudaMemcpyAsync(c->tm_ptr, ptr.data(), ptr.size() * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(c->tm_ent, ent.data(), (size_t)total * sizeof(int2), cudaMemcpyHostToDevice, c->stream));
   return SLLBM_OK;
 }
 
@@ -1313,6 +1317,7 @@ sllbm_status sllbm_adjoint_step(sllbm_ctx* c, const float* lam_in, float* lam_ou
         TRY(dalloc(c, &c->atmp, (size_t)kQ * c->nv));
       }
     }
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));   // (the next call may be on another stream)
     c->transposed = true;
   }
   AdjointArgs a{};
