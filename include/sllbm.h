@@ -276,11 +276,12 @@ sllbm_status sllbm3d_init_equilibrium(sllbm3d_ctx* ctx, const double* rho_dev, c
  * take the sum-factorised step (two launches: TMA-staged tiles that interpolate and sum the moments,
  * a sweep that relaxes and writes the periodic images in the state's ghost cells); the others the
  * one-launch gather step.  The sum-factorised step keeps 2 (orders 1, 2) or 4 ghost cells on every
- * axis in its state and allocates 6 floats a vertex of scratch at sllbm3d_precompute_departures.
+ * axis in its state and 6 floats a vertex of scratch (30 on grids of few tiles); where the device has no
+ * room for that at sllbm3d_create, the grid takes the gather step on a dense state.
  */
 sllbm_status sllbm3d_step(sllbm3d_ctx* ctx, int nsteps);
 /* Name of the kernel sllbm3d_step uses for this context ("stream3d" for the sum-factorised FP32
- * step, "gather_f32", "plain_f64"); valid after sllbm3d_precompute_departures. */
+ * step, "gather_f32", "plain_f64"). */
 const char* sllbm3d_step_kernel_name(const sllbm3d_ctx* ctx);
 /* rho, u, v, w, T of the current state (FP64 device arrays of nz*ny*nx, each may be NULL);
  * synchronises; SLLBM_ERR_UNSTABLE if a step or this call saw a non-positive or non-finite

@@ -44,7 +44,7 @@ struct StepArgs {
   int mapped;           // 1: use descriptors
   // fused uniform kernel geometry
   int offx_min, offx_max, offy_min, offy_max;
-  // optional vertex list (gather kernel only): process vlist[0..nlist) instead of every vertex
+  // optional vertex list (fix-up and gather kernels): process vlist[0..nlist) instead of every vertex
   const int* vlist;
   long long nlist;
   GhostK ghost;         // periodic images to keep up to date in the ghost cells
@@ -57,8 +57,8 @@ struct StepArgs {
   int gx, gy, rows_alloc;
 };
 
-// Cell-periodic pattern of a uniform grid (see step_uniform.cu): per velocity component and
-// local node, the y interpolation as a band of 2p+1 taps around the vertex and the x taps.
+// Cell-periodic pattern of a uniform grid (see step_uniform.cuh): per velocity component and local
+// node, the start of the stencil (a whole cell) and its p + 1 weights, along y and x.
 struct UniformTables {
   bool valid;
   double wy_pat[kQ1][4][5];   // [b][l][alpha]
@@ -100,7 +100,8 @@ struct MappedTables {
 cudaError_t launch_step_mapped(const StepArgs& a, const MappedTables& t, int store, cudaStream_t s);
 size_t mapped_smem_bytes(int bw, int bh, int store);
 
-// Generic FP32 gather step (one thread per vertex, (p+1)^2 gathers per plane from L1/L2).
+// Generic FP32 gather step (one thread per vertex, (p+1)^2 gathers per plane from L1/L2), departures from
+// the descriptors.
 cudaError_t launch_step_gather(const StepArgs& a, int store, cudaStream_t s);
 // Fused shared-memory step for uniform grids (pattern band interpolation); writes only the
 // vertices marked in std_x/std_y, or with t.edge every vertex in two launches.  cudaErrorNotSupported if the tables are not valid.

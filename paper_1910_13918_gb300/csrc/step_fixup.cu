@@ -7,8 +7,8 @@
 // (collide_deviation_f32).
 //
 // What bounds it is latency: the list has one row or column of vertices per clamped side (16
-// vertices on the 8193 x 8 strip, 12,288 on the 3073^2 grid), so a thread per vertex (the gather
-// kernel, 25 dependent gathers and the collision in one thread) left the chip idle for 43 us on
+// vertices on the 8193 x 8 strip, 2,000 at most: more go to the fused kernel's edge tiles), so a thread per
+// vertex (25 dependent gathers and the collision in one thread) left the chip idle for 43 us on
 // that strip, longer than the fused kernel beside it; a warp per vertex has all 25 gathers in
 // flight at once.  The launch overlaps the fused kernel's last tiles (programmatic dependent
 // launch): it reads what that kernel reads, written by steps that ended before it began, and

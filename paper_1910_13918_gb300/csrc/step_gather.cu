@@ -3,14 +3,15 @@
 // the interleaved FP32/BF16 layout: each load brings the (f, g) pair of one (velocity, vertex),
 // and both populations are interpolated together in packed FP32x2 arithmetic.
 //
-// Used for transformed grids (per-(velocity, vertex) departure descriptors, Sec. III.E) and for
-// uniform grids whose departure offsets exceed the staging halo of the fused uniform kernel.
-// Pull streaming of Eq. sl_streaming with the BGK collision of Eq. streaming_fg (Pr = 1).
+// Departures come as per-(velocity, vertex) cells and local coordinates (Sec. III.E): the tiles of
+// transformed grids whose windows the mapped kernel cannot stage, and the uniform grids that the fused
+// kernel does not take (fewer than three cells an axis, departures beyond the neighbouring cells).
+// Pull streaming of Eq. sl_streaming with the BGK collision of Eq. streaming_fg, Pr = 1 or not.
 #include "kernels.h"
 
 namespace sllbm {
 
-template <int P, typename Store, bool Mapped, bool PR>
+template <int P, typename Store, bool PR>
 __global__ void __launch_bounds__(128) step_gather_kernel(const __grid_constant__ StepArgs a) {
   long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (a.vlist) {
@@ -25,24 +26,11 @@ __global__ void __launch_bounds__(128) step_gather_kernel(const __grid_constant_
   float2 fg[kQ];   // (f, g) deviations after streaming
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const int ia = i / 5, ib = i % 5;
-    int sx, sy;
+    const long long d = (long long)i * a.nv + v;
+    const int sx = a.dcx[d] * P, sy = a.dcy[d] * P;
     float wx[P + 1], wy[P + 1];
-    if (Mapped) {
-      const long long d = (long long)i * a.nv + v;
-      sx = a.dcx[d] * P;
-      sy = a.dcy[d] * P;
-      lagrange_basis<P, float>(a.nodesf, a.dr[d], wx);
-      lagrange_basis<P, float>(a.nodesf, a.ds[d], wy);
-    } else {
-      sx = ix + a.offx[ia * a.nx + ix];
-      sy = iy + a.offy[ib * a.ny + iy];
-#pragma unroll
-      for (int k = 0; k <= P; ++k) {
-        wx[k] = a.wx[(ia * a.nx + ix) * (P + 1) + k];
-        wy[k] = a.wy[(ib * a.ny + iy) * (P + 1) + k];
-      }
-    }
+    lagrange_basis<P, float>(a.nodesf, a.dr[d], wx);
+    lagrange_basis<P, float>(a.nodesf, a.ds[d], wy);
     int col[P + 1];
     long long row[P + 1];
 #pragma unroll
@@ -89,10 +77,7 @@ static cudaError_t launch_p(const StepArgs& a, cudaStream_t s) {
   const long long n = a.vlist ? a.nlist : a.nv;
   if (n == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((n + threads - 1) / threads);
-  if (a.mapped)
-    step_gather_kernel<P, Store, true, PR><<<blocks, threads, 0, s>>>(a);
-  else
-    step_gather_kernel<P, Store, false, PR><<<blocks, threads, 0, s>>>(a);
+  step_gather_kernel<P, Store, PR><<<blocks, threads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -108,6 +93,7 @@ static cudaError_t launch_store(const StepArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_step_gather(const StepArgs& a, int store, cudaStream_t s) {
+  if (!a.mapped || !a.dcx) return cudaErrorInvalidValue;
   if (store == kStoreBF16) return launch_store<__nv_bfloat16>(a, s);
   return launch_store<float>(a, s);
 }

@@ -1,14 +1,15 @@
 // Fused SLLBM step for uniform grids, FP32 arithmetic, FP32 or BF16 deviation storage.
 //
 // Pull streaming (Eq. sl_streaming) + moments + fourth-order equilibrium + BGK (Eq. streaming_fg,
-// Pr = 1) in one kernel.  On a uniform grid the departure x_v - dt xi_i separates per axis and,
+// Pr = 1 or not) in one kernel.  On a uniform grid the departure x_v - dt xi_i separates per axis and,
 // away from clamped (zero-gradient) boundaries, repeats with the period p of the cells: the
 // stencil offset and Lagrange weights of vertex j depend only on the velocity component and on
 // the local node j mod p.  The kernel uses that "pattern" (per component and local node: a start
 // offset in [-p, 0] and p+1 weights), for the y interpolation of every staged column and the x
 // interpolation of every vertex.  Vertices whose table entries differ from the pattern (next to
 // zero-gradient boundaries) go to a second launch: the fix-up kernel on exactly those vertices
-// (step_fixup.cu), or on large states the EDGE instance of this kernel on the tiles that hold them.
+// (step_fixup.cu), or on large states and where they are thousands the EDGE instance of this kernel on
+// the tiles that hold them.
 //
 // State: f and g share the departure points, so the state interleaves them ((f, g) pairs per
 // velocity plane and vertex) and every interpolation step moves and combines the pair at once:

@@ -36,7 +36,7 @@ static __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, unsigned par
   return ok != 0;
 }
 // Wait for a phase of an mbarrier with an iteration limit; on timeout set bit 2 of *flag and
-// return false (the kernels then stop their CTA: see step_uniform.cu), so nothing hangs.
+// return false (the kernels then stop their CTA: see step_uniform.cuh), so nothing hangs.
 template <long Limit = (1L << 22)>
 static __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int* flag) {
   for (long it = 0; it < Limit; ++it)
