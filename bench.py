@@ -441,6 +441,8 @@ def measure(w, prec, args, stream, verts, sampler=None, keep=False):
             _barrier()
             ms.append(max_over_ranks(e0.elapsed_time(e1)))
         clocks = sampler.stop() if sampler else None
+        mom = s.moments()   # of the steps so far, for every form and whether kept or not
+        final = torch.stack([mom["rho"], mom["u"], mom["v"], mom["T"]])
         with_moments = None
         if keep and w.velset != "d2q9":   # the same steps with the moments epilogue (D2Q25; 16 B a vertex)
             buf = torch.empty((4, s.ny, s.nx), dtype=torch.float32, device=s.device)
@@ -453,8 +455,6 @@ def measure(w, prec, args, stream, verts, sampler=None, keep=False):
             torch.cuda.synchronize()
             with_moments = max_over_ranks(e0.elapsed_time(e1)) / args.steps
             del buf
-        mom = s.moments()
-        final = torch.stack([mom["rho"], mom["u"], mom["v"], mom["T"]])
         info = {"kernel": s.kernel_name, "launches_per_step": s.launches_per_step,
                 "state_bytes": s.state_bytes, "mass_after": mom["mass"], "nx": s.nx, "ny": s.ny,
                 "precompute_ms": precompute_ms, "ms_per_step_with_moments": with_moments}
