@@ -39,16 +39,23 @@ METRIC = "GVUPS (vertex x velocity x population updates/s), fused FP32 SLLBM ste
 UNIT = "GVUPS"
 SECONDARY = "tgv256"          # second grid of the line: the Taylor-Green vortex, p = 4
 
-# DRAM traffic (read + write bytes per launch) of the step kernel from an ncu capture, keyed by
-# (kernel source digest, workload, precision); reported as null once the kernel source changes.
+# DRAM traffic (bytes a step) of the step kernels, keyed by (kernel source digest, workload, precision);
+# reported as null once the kernel source changes.  Reads from an ncu capture; of the writes a capture counts
+# what has left the L2 when the launch ends, and the rest follows during the next, so every stored value
+# (200 B a vertex) counts once.
+def step_traffic(read, vertices):
+    return read + 200.0 * vertices
+
+
 NCU_TRAFFIC = {
-    # 512^2-cell capture, both launches of a step (interior tiles 484.1 MB read + 415.9 MB written,
-    # edge tiles 38.2 MB read, their writes still in L2), 2,362,369 vertices, scaled by the vertex count
-    # to the 3073^2 grid (a multi-pass capture of that grid exceeds the size rule)
-    ("063a83de6c004d8b", "riemann1024_p3_tableIII", "f32"): 938.24e6 * 9443329 / 2362369,
-    ("063a83de6c004d8b", "riemann512_p3_tableIII", "f32"): 938.24e6,
-    # full-size capture: 217.7 MB read + 170.3 MB written
-    ("063a83de6c004d8b", "tgv256_p4", "f32"): 388.0e6,
+    # 512^2-cell capture, 2,362,369 vertices: interior tiles (2,301,120 vertices) 484.8 MB read (416.1 MB of 460.2
+    # written), 608 edge tiles 38.2 MB read.  The 3073^2 grid (a multi-pass capture of it exceeds the size rule) has
+    # 9,320,640 vertices in interior tiles and 1216 edge tiles.
+    ("05e43b3f4c35dfea", "riemann1024_p3_tableIII", "f32"):
+        step_traffic(484.8e6 * 9320640 / 2301120 + 38.2e6 * 1216 / 608, 9443329),
+    ("05e43b3f4c35dfea", "riemann512_p3_tableIII", "f32"): step_traffic(484.8e6 + 38.2e6, 2362369),
+    # full-size capture: 217.7 MB read (170.0 MB of 209.7 written)
+    ("05e43b3f4c35dfea", "tgv256_p4", "f32"): step_traffic(217.7e6, 1048576),
 }
 
 # Sources that decide what the fused kernels of NCU_TRAFFIC do and how they are launched on

@@ -43,8 +43,8 @@ struct Step3Args {
 
 // Layout of an FP32 pair state: plane i, vertex (x, y, z) at
 // i * plane + origin + (z * rows + y) * pitch + x, with g ghost cells before the interior on
-// every axis (g = 0: the dense [125][nz][ny][nx]; the sum-factorised step keeps g = 2 and the
-// periodic images in the ghost cells, so that its staged regions never wrap).
+// every axis (g = 0: the dense [125][nz][ny][nx]; the sum-factorised step keeps g = 2, or 4 at orders 3
+// and 4, and the periodic images in the ghost cells, so that its staged regions never wrap).
 struct Pad3 {
   int g, pitch, rows;
   size_t plane, origin;
